@@ -9,6 +9,7 @@
 #include "../../include/dirac.h"
 #include "dirac_df.cuh"
 #include "dirac_handle.h"
+#include "dirac_transport.cuh"
 
 using namespace dirac;
 
@@ -261,6 +262,7 @@ dirac_handle::~dirac_handle()
     release(links32);
     release(links_alt);
     release(links_tc);
+    release(scr);
     release(ws_in);
     release(ws_out);
     free_solver_workspace();
@@ -335,13 +337,24 @@ dirac_status dirac_set_links(dirac_handle* h, const void* V, dirac_prec V_prec, 
     if (!h->links && (st = h->alloc(&h->links, nblk_of((size_t)h->g.vol) * 32 * 9 * nmat * cbytes(h->prec), "links")))
         return st;
     if (h->op == OP_BRILLOUIN) {
-        if ((st = h->build_W64())) return st;
-        st = h->cuda(launch_convert_links(h->prec, h->g, 40, h->W64, h->links, h->stream), "W conversion");
+        if (h->prec == P_F64) {
+            if ((st = h->build_W64())) return st;
+            st = h->cuda(launch_convert_links(h->prec, h->g, 40, h->W64, h->links, h->stream), "W conversion");
+        } else {
+            // W rounded to FP32 or less: built in double-float (the solver builds FP64 W on demand)
+            void* W = nullptr;
+            if ((st = h->scratch((size_t)h->g.vol * 40 * 9 * 16, &W))) return st;
+            st = h->cuda(launch_build_W(h->g, h->links64, W, true, h->stream), "W build");
+            if (!st) st = h->cuda(launch_convert_links_df(h->prec, h->g, 40, W, h->links, h->stream), "W conversion");
+            // the FP32 copy of the split inner solve is refreshed in place (a
+            // captured solver graph holds its address)
+            if (!st && h->links32 && h->links32 != h->links) {
+                st = h->cuda(launch_convert_links_df(P_F32, h->g, 40, W, h->links32, h->stream), "FP32 W (blocked)");
+                if (!st) st = h->cuda(launch_brillouin_w80(P_F32, h->g, h->links32, h->links32, h->stream), "FP32 W, 80 directions");
+            }
+            h->scratch_done();
+        }
         if (st) return st;
-        // the FP32 copy of the split inner solve is refreshed in place (a
-        // captured solver graph holds its address)
-        if (h->links32 && h->links32 != h->links && (st = h->refresh_links32())) return st;
-        if (h->prec != P_F64) h->release_after_sync(h->W64);   // rebuilt on demand by the solver
     } else {
         st = h->cuda(launch_convert_links(h->prec, h->g, 4, h->links64, h->links, h->stream), "links conversion");
         if (st) return st;
@@ -482,15 +495,37 @@ dirac_status dirac_handle::build_W64()
 {
     if (W64) return DIRAC_OK;
     dirac_status st;
-    void* tmp = nullptr;
-    if ((st = alloc(&tmp, (size_t)g.vol * 81 * 9 * 16, "W build scratch"))) return st;
-    if ((st = alloc(&W64, (size_t)g.vol * 40 * 9 * 16, "FP64 W"))) {
-        release(tmp);
-        return st;
-    }
-    st = cuda(launch_build_W(g, links64, tmp, W64, stream), "W build");
-    release_after_sync(tmp);
+    if ((st = alloc(&W64, (size_t)g.vol * 40 * 9 * 16, "FP64 W"))) return st;
+    st = cuda(launch_build_W(g, links64, W64, false, stream), "W build");
+    if (st) release_after_sync(W64);
     return st;
+}
+
+// scratch of the W build and of the Brillouin link gradient (17 KB per site).
+// Up to SCRATCH_KEEP bytes stay with the handle for the next call: allocating
+// and freeing 0.5 GB took 1.4 ms of a 2.6 ms gradient (12^3 x 16).  A larger one is
+// given back after the call.  scratch_done waits for the stream, so a later
+// call may use the memory on another one.
+dirac_status dirac_handle::scratch(size_t bytes, void** out)
+{
+    if (bytes > scr_bytes) {
+        release(scr);
+        scr_bytes = 0;
+        dirac_status st = alloc(&scr, bytes, "Brillouin transporter scratch");
+        if (st) return st;
+        scr_bytes = bytes;
+    }
+    *out = scr;
+    return DIRAC_OK;
+}
+
+void dirac_handle::scratch_done()
+{
+    cudaStreamSynchronize(stream);
+    if (scr_bytes > SCRATCH_KEEP) {
+        release(scr);
+        scr_bytes = 0;
+    }
 }
 
 void dirac_handle::release_after_sync(void*& p)

@@ -146,18 +146,15 @@ extern "C" DIRAC_API dirac_status dirac_force(dirac_handle* h, void* F, const vo
         gi = h->ws_out;
     }
     if (h->op == OP_BRILLOUIN) {
-        // the transporters are rebuilt from V in FP64 (not kept from the forward pass)
-        void *w81 = nullptr, *g81 = nullptr;
-        const size_t fb = (size_t)h->g.vol * 81 * 9 * 16;
-        if ((st = h->alloc(&w81, fb, "Brillouin force scratch"))) return st;
-        if ((st = h->alloc(&g81, fb, "Brillouin force scratch"))) {
-            h->release(w81);
-            return st;
-        }
-        st = h->cuda(launch_force_brillouin(h->prec, h->g, h->Nv, pi, gi, h->links64, w81, g81, F, h->stream),
+        // the transporters are rebuilt from V (not kept from the forward pass):
+        // 40 planes of W and 81 of G
+        const size_t plane = (size_t)h->g.vol * 9 * 16;
+        void* scr = nullptr;
+        if ((st = h->scratch(121 * plane, &scr))) return st;
+        st = h->cuda(launch_force_brillouin(h->prec, h->g, h->Nv, pi, gi, h->links64, scr,
+                                            static_cast<char*>(scr) + 40 * plane, F, h->stream),
                      "Brillouin force kernels");
-        h->release_after_sync(w81);
-        h->release_after_sync(g81);
+        h->scratch_done();
         return st;
     }
     return h->cuda(launch_force(h->op, h->prec, h->g, h->Nv, pi, gi, F, h->stream), "force kernel launch");

@@ -9,84 +9,113 @@
 // Steps (all gathers, one write per output element, no atomics):
 //   1. G_dir(y) = dL/dW_dir(y) = sum_{v,s} g_v(y)_s (M_dir psi_v(y+dir))_s^+
 //      for the 80 directions, M_dir = rho_k (dir . gamma) - lambda_k / 2;
-//   (every step in FP64 arithmetic, whatever the storage precision)
 //   2. for k = 4, 3, 2 the (k-1)-hop gradients collect what the k-hop
 //      directions pass down: G_{d'}(y) += (1/k) H_a(y-a)^+ G_{d'+a}(y-a) over
 //      the hops a on the axes d' does not use;
 //   3. F_mu(y) = sum_{dir with +mu} (1/k) G_dir(y) W_{dir-mu}(y+mu)^+
 //             + sum_{dir with -mu} (1/k) W_{dir+mu}(y) G_dir(y+mu)^+
 //      (W_0 = 1: the one-hop directions).
+// Arithmetic: FP64 for FP64 handles; for the others, whose psi and g are exact
+// in FP32 and whose F is rounded to FP32, double-float (dirac_transport.cuh).
+// All steps are bound by arithmetic (step 1: 36 complex multiply-adds per
+// direction and right-hand side, 144 FP64 operations, at a sixtieth of the
+// FP32 rate); 12^3 x 16, 8 right-hand sides, FP32 storage, one GB300:
+//                 FP64      double-float
+//   step 1        9.51 ms   1.43 ms
+//   W build       1.12 ms   0.28 ms  (80 directions in FP64, 40 here)
+//   step 2        1.26 ms   0.56 ms
+//   step 3        1.42 ms   0.54 ms
 #include "dirac_handle.h"
 #include "dirac_kernels.cuh"
+#include "dirac_transport.cuh"
 
 using namespace dirac;
 
 namespace dirac {
 namespace {
 
-__device__ __forceinline__ void dir_of(int c, int d[4])
-{
-    d[0] = c % 3 - 1;
-    d[1] = (c / 3) % 3 - 1;
-    d[2] = (c / 9) % 3 - 1;
-    d[3] = (c / 27) % 3 - 1;
-}
-__device__ __forceinline__ int code_of(const int d[4])
-{
-    return (d[0] + 1) + 3 * (d[1] + 1) + 9 * (d[2] + 1) + 27 * (d[3] + 1);
-}
+// h_s of the spin-transformed g: h = (M_dir / rho_k) g = kappa g + (dir . gamma) g with
+// kappa = -lambda_k / (2 rho_k) = -27 2^(k-7), exact in FP32; M_dir is hermitian, so
+// sum_s g_s (M psi)_s^+ = sum_s (M g)_s psi_s^+, and moving it from psi to g leaves one
+// transform by sums of signed components; rho_k goes into the final scale of G.
+// chiral basis, (gamma_mu g)_s = phase g_sigma: x: s <-> 3 - s, phases -i -i i i;
+// y: s <-> 3 - s, - + + -; z: s <-> s ^ 2, -i i i -i; t: s <-> s ^ 2, 1
+// sums of FP32 components in (hi, lo), exact up to the last bits of lo
+struct Sum2 {
+    float hi, lo;
+    __device__ __forceinline__ void start(float kappa, float g)
+    {
+        hi = df_mul(kappa, g);
+        lo = df_fma(kappa, g, -hi);
+    }
+    __device__ __forceinline__ void add(float t)
+    {
+        float s, e;
+        dd::two_sum(hi, t, s, e);
+        hi = s;
+        lo = df_add(lo, e);
+    }
+    __device__ __forceinline__ dfl get() const { return dfl(hi, lo); }
+};
+struct Sum1 {
+    double v;
+    __device__ __forceinline__ void start(double kappa, double g) { v = kappa * g; }
+    __device__ __forceinline__ void add(double t) { v += t; }
+    __device__ __forceinline__ double get() const { return v; }
+};
 
-// the spin matrix of direction d: [[a, rho Q], [rho Q^+, a]], a = -lambda_k / 2,
-// Q = sum_mu d_mu B_mu (B_k = -i sigma_k, B_4 = 1); rho_k, lambda_k of Sec. 5
-template <typename A>
-__device__ __forceinline__ BriDirA<A> coeffs_of(const int d[4])
-{
-    const int k = abs(d[0]) + abs(d[1]) + abs(d[2]) + abs(d[3]);
-    const double rho[5] = {0.0, 64.0 / 432.0, 16.0 / 432.0, 4.0 / 432.0, 1.0 / 432.0};
-    const double lam[5] = {-240.0 / 64.0, 8.0 / 64.0, 4.0 / 64.0, 2.0 / 64.0, 1.0 / 64.0};
-    const double r = rho[k];
-    const double dx = d[0], dy = d[1], dz = d[2], dt = d[3];
-    BriDirA<A> m;
-    m.a = (A)(-0.5 * lam[k]);
-    m.q00 = {(A)(r * dt), (A)(-r * dz)};
-    m.q01 = {(A)(-r * dy), (A)(-r * dx)};
-    m.q10 = {(A)(r * dy), (A)(-r * dx)};
-    m.q11 = {(A)(r * dt), (A)(r * dz)};
-    return m;
-}
-
-__device__ __forceinline__ cx<double> ld64(const double2* p, size_t i)
-{
-    const double2 v = p[i];
-    return {v.x, v.y};
-}
-
-// C = A B, A^+ B, A B^+ (3x3)
-__device__ __forceinline__ void mm(const cx<double>* Am, bool adag, const cx<double>* Bm, bool bdag, cx<double>* C)
+template <typename A, typename S>
+__device__ __forceinline__ void h_spin(int s, const int (&d)[4], A kappa, const cx<A>* g, S (&re)[3], S (&im)[3])
 {
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
+    for (int c = 0; c < 3; ++c) {
+        re[c].start(kappa, g[3 * s + c].re);
+        im[c].start(kappa, g[3 * s + c].im);
+    }
+    const cx<A>* gx = g + 3 * (3 - s);
+    const cx<A>* gz = g + 3 * (s ^ 2);
+    if (d[0]) {   // uniform over the warp: all its threads work on one direction
+        const A f = (s < 2) ? A(d[0]) : A(-d[0]);   // -i f g
 #pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            cx<double> t{0.0, 0.0};
-#pragma unroll
-            for (int m = 0; m < 3; ++m) {
-                const cx<double> x = adag ? conj(Am[3 * m + a]) : Am[3 * a + m];
-                const cx<double> y = bdag ? conj(Bm[3 * b + m]) : Bm[3 * m + b];
-                t = cfma(x, y, t);
-            }
-            C[3 * a + b] = t;
+        for (int c = 0; c < 3; ++c) {
+            re[c].add(f * gx[c].im);
+            im[c].add(-f * gx[c].re);
         }
+    }
+    if (d[1]) {
+        const A f = (s == 0 || s == 3) ? A(-d[1]) : A(d[1]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            re[c].add(f * gx[c].re);
+            im[c].add(f * gx[c].im);
+        }
+    }
+    if (d[2]) {
+        const A f = (s == 0 || s == 3) ? A(d[2]) : A(-d[2]);   // -i f g
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            re[c].add(f * gz[c].im);
+            im[c].add(-f * gz[c].re);
+        }
+    }
+    if (d[3]) {
+        const A f = A(d[3]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            re[c].add(f * gz[c].re);
+            im[c].add(f * gz[c].im);
+        }
+    }
 }
 
-// step 1: one thread per (site, direction j = 0..79).  The arithmetic is FP64
-// for every storage precision: FP32 and 16-bit values are exact in FP64, so
-// G is the FP64 gradient of the stored psi and g (the steps below are FP64
-// as well), and F is rounded once, at its store.
+// step 1: one thread per (site, direction j = 0..79)
 template <typename T>
-__global__ void __launch_bounds__(128) k_bri_gradW(Geom g, int Nv, const void* psi, const void* gv, double2* G81)
+__global__ void __launch_bounds__(128) k_bri_gradW(Geom g, int Nv, const void* psi, const void* gv, void* G81)
 {
-    using A = typename Store<T>::A;
+    using A = typename Store<T>::A;                                                // of psi and g
+    constexpr bool F64 = sizeof(A) == 8;
+    using B = typename std::conditional<F64, double, dfl>::type;                   // of G
+    using S = typename std::conditional<F64, Sum1, Sum2>::type;
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;   // (site, j), site fastest
     if (i >= 80 * g.vol) return;
     const long y = i % g.vol;
@@ -98,93 +127,91 @@ __global__ void __launch_bounds__(128) k_bri_gradW(Geom g, int Nv, const void* p
     int x[4];
     site_offsets(g, y, fwd, bwd, x);
     long nb = y;
+    int k = 0;
 #pragma unroll
-    for (int mu = 0; mu < 4; ++mu) nb += d[mu] > 0 ? fwd[mu] : (d[mu] < 0 ? bwd[mu] : 0);
-    const BriDirA<double> m = coeffs_of<double>(d);
-    cx<double> acc[9];
+    for (int mu = 0; mu < 4; ++mu) {
+        nb += d[mu] > 0 ? fwd[mu] : (d[mu] < 0 ? bwd[mu] : 0);
+        k += d[mu] != 0;
+    }
+    const A kappa = A(-27.0 / 64.0) * A(1 << (k - 1));
+    cx<B> acc[9];
 #pragma unroll
-    for (int e = 0; e < 9; ++e) acc[e] = cx<double>{0.0, 0.0};
+    for (int e = 0; e < 9; ++e) acc[e] = cx<B>{B(0), B(0)};
     for (int v = 0; v < Nv; ++v) {
         cx<A> ps[12], gs[12];
         load_spinor<T, 12>(psi, g.vol, v, nb, ps);
         load_spinor<T, 12>(gv, g.vol, v, y, gs);
-        cx<double> p[12], chi[12], gg[12];
 #pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            p[k] = cx<double>{(double)ps[k].re, (double)ps[k].im};
-            gg[k] = cx<double>{(double)gs[k].re, (double)gs[k].im};
+        for (int s = 0; s < 4; ++s) {
+            S hr[3], hi[3];
+            h_spin<A, S>(s, d, kappa, gs, hr, hi);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const cx<B> h{hr[a].get(), hi[a].get()};
+#pragma unroll
+                for (int b = 0; b < 3; ++b) cmacc_conj(h, ps[3 * s + b], acc[3 * a + b]);
+            }
         }
-        bri_spin(m, p, chi);
-#pragma unroll
-        for (int s = 0; s < 4; ++s)
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-#pragma unroll
-                for (int b = 0; b < 3; ++b) acc[3 * a + b] = cfma_conj(chi[3 * s + b], gg[3 * s + a], acc[3 * a + b]);
     }
+    const B rho = B((double)(1 << (8 - 2 * k)) / 432.0);
 #pragma unroll
-    for (int e = 0; e < 9; ++e) G81[((size_t)c * 9 + e) * g.vol + y] = make_double2(acc[e].re, acc[e].im);
+    for (int e = 0; e < 9; ++e)
+        st_el(G81, ((size_t)c * 9 + e) * g.vol + y, cx<B>{times(settle(acc[e].re), rho), times(settle(acc[e].im), rho)});
 }
 
-struct Codes {
-    int n;
-    short c[32];
-};
-
 // step 2 for level k: one thread per (site, direction of k-1 hops)
-__global__ void __launch_bounds__(128) k_bri_back(Geom g, Codes L, int k, const double2* __restrict__ V64,
-                                                  double2* G81)
+template <typename A>
+__global__ void __launch_bounds__(128) k_bri_back(Geom g, const __grid_constant__ DirList L, const __grid_constant__ DirPlanes P, int k, const void* W, void* G81)
 {
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long)L.n * g.vol) return;
     const long y = i % g.vol;
-    const int c = L.c[i / g.vol];
+    const int c = L.code[i / g.vol];
     int d[4];
     dir_of(c, d);
     long fwd[4], bwd[4];
     int x[4];
     site_offsets(g, y, fwd, bwd, x);
-    cx<double> Gs[9];
+    cx<A> acc[9];
 #pragma unroll
-    for (int e = 0; e < 9; ++e) Gs[e] = ld64(G81, ((size_t)c * 9 + e) * g.vol + y);
-    const double inv = 1.0 / k;
+    for (int e = 0; e < 9; ++e) acc[e] = cx<A>{A(0), A(0)};
+#pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
         if (d[mu] != 0) continue;
-        cx<double> U[9], Gu[9], T9[9];
-        // a = +mu: (1/k) V_mu(y-mu)^+ G_{d+mu}(y-mu)
-        int dp[4] = {d[0], d[1], d[2], d[3]};
-        dp[mu] = 1;
-        const long sm = y + bwd[mu];
-        const int cp = code_of(dp);
-#pragma unroll
-        for (int e = 0; e < 9; ++e) {
-            U[e] = ld64(V64, ((size_t)mu * 9 + e) * g.vol + sm);
-            Gu[e] = ld64(G81, ((size_t)cp * 9 + e) * g.vol + sm);
+        const int e1[4] = {mu == 0, mu == 1, mu == 2, mu == 3};
+        const int pv = P.p[code_of(e1)];   // the plane of V_mu
+        cx<A> U[9], Gu[9];
+        // a = +mu: V_mu(y-mu)^+ G_{d+mu}(y-mu);  a = -mu: V_mu(y) G_{d-mu}(y+mu)
+#pragma unroll 1
+        for (int up = 1; up >= -1; up -= 2) {
+            int dp[4] = {d[0], d[1], d[2], d[3]};
+            dp[mu] = up;
+            const long sn = y + (up > 0 ? bwd[mu] : fwd[mu]);
+            load_mat<A>(W, g.vol, pv, up > 0 ? sn : y, up > 0, U);
+            load_mat<A>(G81, g.vol, code_of(dp), sn, false, Gu);
+            mm_acc(U, Gu, acc);
         }
-        mm(U, true, Gu, false, T9);
-#pragma unroll
-        for (int e = 0; e < 9; ++e) Gs[e] = Gs[e] + scale(inv, T9[e]);
-        // a = -mu: (1/k) V_mu(y) G_{d-mu}(y+mu)
-        dp[mu] = -1;
-        const long sp = y + fwd[mu];
-        const int cm = code_of(dp);
-#pragma unroll
-        for (int e = 0; e < 9; ++e) {
-            U[e] = ld64(V64, ((size_t)mu * 9 + e) * g.vol + y);
-            Gu[e] = ld64(G81, ((size_t)cm * 9 + e) * g.vol + sp);
-        }
-        mm(U, false, Gu, false, T9);
-#pragma unroll
-        for (int e = 0; e < 9; ++e) Gs[e] = Gs[e] + scale(inv, T9[e]);
     }
+    const A inv = A(1.0 / k);
 #pragma unroll
-    for (int e = 0; e < 9; ++e) G81[((size_t)c * 9 + e) * g.vol + y] = make_double2(Gs[e].re, Gs[e].im);
+    for (int e = 0; e < 9; ++e) {
+        const size_t o = ((size_t)c * 9 + e) * g.vol + y;
+        const cx<A> G0 = ld_el<A>(G81, o);
+        st_el(G81, o, cx<A>{plus(G0.re, times(settle(acc[e].re), inv)), plus(G0.im, times(settle(acc[e].im), inv))});
+    }
 }
 
+// the directions with a hop along mu, ordered by their number of hops
+struct DirsOfMu {
+    short code[4][54];
+};
+
+__device__ __forceinline__ float as_out(dfl a) { return a.hi; }
+__device__ __forceinline__ double as_out(double a) { return a; }
+
 // step 3: one thread per (site, mu); F canonical [site][mu][a][b] in the type O
-template <typename O>
-__global__ void __launch_bounds__(128) k_bri_dV(Geom g, const double2* __restrict__ G81,
-                                                const double2* __restrict__ W81, O* F)
+template <typename A, typename O>
+__global__ void __launch_bounds__(128) k_bri_dV(Geom g, const __grid_constant__ DirsOfMu D, const __grid_constant__ DirPlanes P, const void* G81, const void* W, O* F)
 {
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;   // (site, mu), site fastest
     if (i >= 4 * g.vol) return;
@@ -193,76 +220,106 @@ __global__ void __launch_bounds__(128) k_bri_dV(Geom g, const double2* __restric
     long fwd[4], bwd[4];
     int x[4];
     site_offsets(g, y, fwd, bwd, x);
-    const long yp = y + fwd[mu];
-    cx<double> acc[9];
+    long fm = fwd[0];
 #pragma unroll
-    for (int e = 0; e < 9; ++e) acc[e] = cx<double>{0.0, 0.0};
-    for (int c = 0; c < 81; ++c) {
-        int d[4];
-        dir_of(c, d);
-        if (d[mu] == 0) continue;
-        const int k = abs(d[0]) + abs(d[1]) + abs(d[2]) + abs(d[3]);
-        const double inv = 1.0 / k;
-        int r[4] = {d[0], d[1], d[2], d[3]};
-        r[mu] = 0;
-        const int cr = code_of(r);
-        cx<double> Gm[9], Wr[9], T9[9];
-        if (d[mu] > 0) {
-            // (1/k) G_dir(y) W_{dir-mu}(y+mu)^+
+    for (int nu = 1; nu < 4; ++nu)
+        if (mu == nu) fm = fwd[nu];
+    const long yp = y + fm;
+    cx<A> F9[9];
 #pragma unroll
-            for (int e = 0; e < 9; ++e) Gm[e] = ld64(G81, ((size_t)c * 9 + e) * g.vol + y);
+    for (int e = 0; e < 9; ++e) F9[e] = cx<A>{A(0), A(0)};
+    int j = 0;
+#pragma unroll 1
+    for (int k = 1; k <= 4; ++k) {
+        const int nk = k == 1 ? 2 : (k == 2 ? 12 : (k == 3 ? 24 : 16));
+        cx<A> acc[9];
+#pragma unroll
+        for (int e = 0; e < 9; ++e) acc[e] = cx<A>{A(0), A(0)};
+#pragma unroll 1
+        for (int n = 0; n < nk; ++n, ++j) {
+            const int c = D.code[mu][j];
+            int d[4];
+            dir_of(c, d);
+            const int dm = mu == 0 ? d[0] : (mu == 1 ? d[1] : (mu == 2 ? d[2] : d[3]));
+            // dir with +mu: G_dir(y) W_rest(y+mu)^+;  with -mu: W_rest(y) G_dir(y+mu)^+;
+            // rest = dir without its hop along mu
+            cx<A> Gm[9], Wr[9];
+            load_mat<A>(G81, g.vol, c, dm > 0 ? y : yp, dm < 0, Gm);
             if (k == 1) {
 #pragma unroll
-                for (int e = 0; e < 9; ++e) T9[e] = Gm[e];
-            } else {
-#pragma unroll
-                for (int e = 0; e < 9; ++e) Wr[e] = ld64(W81, ((size_t)cr * 9 + e) * g.vol + yp);
-                mm(Gm, false, Wr, true, T9);
+                for (int e = 0; e < 9; ++e) acc[e] = cx<A>{plus(acc[e].re, Gm[e].re), plus(acc[e].im, Gm[e].im)};
+                continue;
             }
-        } else {
-            // (1/k) W_{dir+mu}(y) G_dir(y+mu)^+
+            long so = 0;   // offset of rest
 #pragma unroll
-            for (int e = 0; e < 9; ++e) Gm[e] = ld64(G81, ((size_t)c * 9 + e) * g.vol + yp);
-            if (k == 1) {
-#pragma unroll
-                for (int a = 0; a < 3; ++a)
-#pragma unroll
-                    for (int b = 0; b < 3; ++b) T9[3 * a + b] = conj(Gm[3 * b + a]);
-            } else {
-#pragma unroll
-                for (int e = 0; e < 9; ++e) Wr[e] = ld64(W81, ((size_t)cr * 9 + e) * g.vol + y);
-                mm(Wr, false, Gm, true, T9);
-            }
+            for (int nu = 0; nu < 4; ++nu)
+                if (nu != mu) so += d[nu] > 0 ? fwd[nu] : (d[nu] < 0 ? bwd[nu] : 0);
+            const int p3 = mu == 0 ? 1 : (mu == 1 ? 3 : (mu == 2 ? 9 : 27));
+            const int pr = P.p[c - dm * p3];
+            const long z = dm > 0 ? yp : y;
+            // W_rest(z) or its adjoint; rest not stored: W_rest(z) = W_{-rest}(z + rest)^+
+            load_mat<A>(W, g.vol, pr >= 0 ? pr : -1 - pr, pr >= 0 ? z : z + so, (dm > 0) == (pr >= 0), Wr);
+            if (dm > 0) mm_acc(Gm, Wr, acc);
+            else mm_acc(Wr, Gm, acc);
         }
+        const A inv = A(1.0 / k);
 #pragma unroll
-        for (int e = 0; e < 9; ++e) acc[e] = acc[e] + scale(inv, T9[e]);
+        for (int e = 0; e < 9; ++e)
+            F9[e] = cx<A>{plus(F9[e].re, times(settle(acc[e].re), inv)),
+                           plus(F9[e].im, times(settle(acc[e].im), inv))};
     }
     O* out = F + ((size_t)y * 4 + mu) * 9;
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
         O o;
-        o.x = acc[e].re;
-        o.y = acc[e].im;
+        o.x = as_out(F9[e].re);
+        o.y = as_out(F9[e].im);
         out[e] = o;
     }
 }
 
 template <typename T>
-cudaError_t gradW_T(const Geom& g, int Nv, const void* psi, const void* gv, double2* G81, cudaStream_t st)
+cudaError_t gradW_T(const Geom& g, int Nv, const void* psi, const void* gv, void* G81, cudaStream_t st)
 {
     const long n = 80 * g.vol;
     k_bri_gradW<T><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(g, Nv, psi, gv, G81);
     return cudaGetLastError();
 }
 
+template <typename A, typename O>
+cudaError_t chain_T(const Geom& g, const void* W, void* G, void* F, cudaStream_t st)
+{
+    const DirPlanes P = dir_planes();
+    for (int k = 4; k >= 2; --k) {
+        const DirList L = dirs_of_hops(k - 1, false);
+        const long n = (long)L.n * g.vol;
+        k_bri_back<A><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(g, L, P, k, W, G);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    DirsOfMu D;
+    int n[4] = {0, 0, 0, 0};
+    for (int k = 1; k <= 4; ++k) {
+        const DirList L = dirs_of_hops(k, false);
+        for (int m = 0; m < L.n; ++m) {
+            int d[4];
+            dir_of(L.code[m], d);
+            for (int mu = 0; mu < 4; ++mu)
+                if (d[mu]) D.code[mu][n[mu]++] = L.code[m];
+        }
+    }
+    const unsigned nb = (unsigned)((4 * g.vol + 127) / 128);
+    k_bri_dV<A, O><<<nb, 128, 0, st>>>(g, D, P, G, W, static_cast<O*>(F));
+    return cudaGetLastError();
+}
+
 }   // namespace
 
 cudaError_t launch_force_brillouin(int prec, const Geom& g, int Nv, const void* psi, const void* gv,
-                                   const void* V64, void* W81, void* G81, void* F, cudaStream_t st)
+                                   const void* V64, void* W, void* G, void* F, cudaStream_t st)
 {
-    cudaError_t e = launch_build_W81(g, V64, W81, st);
+    cudaError_t e = launch_build_W(g, V64, W, prec != P_F64, st);
     if (e != cudaSuccess) return e;
-    double2* G = static_cast<double2*>(G81);
     switch (prec) {
     case P_F64: e = gradW_T<double>(g, Nv, psi, gv, G, st); break;
     case P_F32: e = gradW_T<float>(g, Nv, psi, gv, G, st); break;
@@ -271,24 +328,7 @@ cudaError_t launch_force_brillouin(int prec, const Geom& g, int Nv, const void* 
     default: return cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return e;
-    for (int k = 4; k >= 2; --k) {
-        Codes L;
-        L.n = 0;
-        for (int c = 0; c < 81; ++c) {
-            const int d0 = c % 3 - 1, d1 = (c / 3) % 3 - 1, d2 = (c / 9) % 3 - 1, d3 = (c / 27) % 3 - 1;
-            if ((d0 != 0) + (d1 != 0) + (d2 != 0) + (d3 != 0) == k - 1) L.c[L.n++] = (short)c;
-        }
-        const long n = (long)L.n * g.vol;
-        k_bri_back<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(g, L, k, static_cast<const double2*>(V64), G);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    const unsigned nb = (unsigned)((4 * g.vol + 127) / 128);
-    if (prec == P_F64)
-        k_bri_dV<double2><<<nb, 128, 0, st>>>(g, G, static_cast<const double2*>(W81), static_cast<double2*>(F));
-    else
-        k_bri_dV<float2><<<nb, 128, 0, st>>>(g, G, static_cast<const double2*>(W81), static_cast<float2*>(F));
-    return cudaGetLastError();
+    return prec == P_F64 ? chain_T<double, double2>(g, W, G, F, st) : chain_T<dfl, float2>(g, W, G, F, st);
 }
 
 }  // namespace dirac

@@ -44,6 +44,10 @@ struct dirac_handle {
     void* ws_out = nullptr;
     size_t ws_bytes = 0;
 
+    static constexpr size_t SCRATCH_KEEP = (size_t)1 << 30;
+    void* scr = nullptr;      // scratch of the W build and the Brillouin link gradient
+    size_t scr_bytes = 0;
+
     // solver workspace (dirac_solve.cu)
     void* sw = nullptr;
     size_t sw_bytes = 0;
@@ -66,6 +70,8 @@ struct dirac_handle {
     double diag_of(double mass) const;
     dirac_status ensure_workspace();
     dirac_status build_W64();
+    dirac_status scratch(size_t bytes, void** out);
+    void scratch_done();
     dirac_status ensure_links64b(const void** out);
     dirac_status ensure_links_df(const void** out);
     dirac_status ensure_links32(const void** out);

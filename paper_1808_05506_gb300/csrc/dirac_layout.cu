@@ -1,6 +1,6 @@
 // Layout conversion (canonical <-> internal blocked layout) and the
 // Brillouin off-axis link build of Tab. tab:off-axis.
-#include "dirac_internal.h"
+#include "dirac_transport.cuh"
 
 namespace dirac {
 
@@ -229,135 +229,109 @@ cudaError_t launch_convert_links(int prec, const Geom& g, int nmat, const void* 
     return cudaGetLastError();
 }
 
+// double-float links [m][e][site] -> storage precision (FP32 or 16 bits): the
+// high half is the value rounded to FP32
+template <typename T>
+__global__ void k_convert_links_df(long vol, long n, const float4* __restrict__ src, void* dst)
+{
+    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;   // (m, e, site), site fastest
+    if (i >= n) return;
+    const long s = i % vol;
+    const long me = i / vol;
+    const float4 v = src[i];
+    st_one<T>(dst, blk_index((size_t)vol, 9, (int)(me / 9), (int)(me % 9), s), cx<float>{v.x, v.z});
+}
+
+cudaError_t launch_convert_links_df(int prec, const Geom& g, int nmat, const void* src, void* dst, cudaStream_t st)
+{
+    const long n = g.vol * 9L * nmat;
+    const unsigned nb = (unsigned)((n + 255) / 256);
+    const float4* s = (const float4*)src;
+    switch (prec) {
+    case P_F32: k_convert_links_df<float><<<nb, 256, 0, st>>>(g.vol, n, s, dst); break;
+    case P_BF16: k_convert_links_df<__nv_bfloat16><<<nb, 256, 0, st>>>(g.vol, n, s, dst); break;
+    case P_F16: k_convert_links_df<__half><<<nb, 256, 0, st>>>(g.vol, n, s, dst); break;
+    default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
 // ---------------------------------------------------------------- W build
 // Tab. tab:off-axis defines W_dir(x) as the average of the path products over
 // the k! orderings of the k unit hops of dir.  Splitting off the first hop a
 // gives the recursion W_dir(x) = (1/k) sum_{hops a of dir} V_a(x) W_{dir-a}(x+a)
 // with V_{-mu}(x) = V_mu(x-mu)^+; it is evaluated level by level (k = 1..4)
-// in FP64 over all 80 directions, with tmp81 laid out [dir81][9][site].
-__device__ __forceinline__ int dir81_of(const int d[4])
+// for the 40 stored directions, the others being read as adjoints.
+// Bound by arithmetic: 104 products of 3x3 matrices per site.  FP64 handles
+// take FP64; the others double-float, since their W is rounded to FP32 or 16
+// bits (12^3 x 16: 1.12 ms for 80 directions in FP64, 0.28 ms for these).
+template <typename A>
+__global__ void k_w_level1(Geom g, const __grid_constant__ DirPlanes P, const double2* __restrict__ V64, void* W)
 {
-    return (d[0] + 1) + 3 * (d[1] + 1) + 9 * (d[2] + 1) + 27 * (d[3] + 1);
+    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;   // (mu, e, site), site fastest
+    if (i >= g.vol * 36) return;
+    const long s = i % g.vol;
+    const int me = (int)(i / g.vol), mu = me / 9, e = me % 9;
+    int d[4] = {mu == 0, mu == 1, mu == 2, mu == 3};
+    const double2 v = V64[i];
+    st_el(W, ((size_t)P.p[code_of(d)] * 9 + e) * g.vol + s, cx<A>{A(v.x), A(v.y)});
 }
 
-__global__ void k_wbuild_level1(Geom g, const double2* __restrict__ V64, double2* tmp)
-{
-    const long s = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= g.vol) return;
-    long fwd[4], bwd[4];
-    int x[4];
-    site_offsets(g, s, fwd, bwd, x);
-    for (int mu = 0; mu < 4; ++mu) {
-        int dp[4] = {0, 0, 0, 0}, dm[4] = {0, 0, 0, 0};
-        dp[mu] = 1;
-        dm[mu] = -1;
-        const int cp = dir81_of(dp), cm = dir81_of(dm);
-        for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b) {
-                tmp[((size_t)cp * 9 + a * 3 + b) * g.vol + s] = V64[((size_t)mu * 9 + a * 3 + b) * g.vol + s];
-                double2 u = V64[((size_t)mu * 9 + b * 3 + a) * g.vol + s + bwd[mu]];
-                tmp[((size_t)cm * 9 + a * 3 + b) * g.vol + s] = make_double2(u.x, -u.y);
-            }
-    }
-}
-
-struct DirList {
-    int n;
-    int k;
-    short code[32];
-};
-
-__global__ void k_wbuild_level(Geom g, DirList L, double2* tmp)
+template <typename A>
+__global__ void __launch_bounds__(128) k_w_level(Geom g, const __grid_constant__ DirList L, const __grid_constant__ DirPlanes P, void* W)
 {
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;   // (site, j), site fastest
     if (i >= g.vol * L.n) return;
     const long s = i % g.vol;
-    const int j = (int)(i / g.vol);
-    const int c = L.code[j];
-    int d[4] = {c % 3 - 1, (c / 3) % 3 - 1, (c / 9) % 3 - 1, (c / 27) % 3 - 1};
+    const int c = L.code[i / g.vol];
+    int d[4];
+    dir_of(c, d);
     long fwd[4], bwd[4];
     int x[4];
     site_offsets(g, s, fwd, bwd, x);
-    cx<double> acc[9];
-    for (int e = 0; e < 9; ++e) acc[e] = cx<double>{0.0, 0.0};
+    long sd = s;   // x + dir
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) sd += d[mu] > 0 ? fwd[mu] : (d[mu] < 0 ? bwd[mu] : 0);
+    cx<A> acc[9];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) acc[e] = cx<A>{A(0), A(0)};
+#pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
         if (d[mu] == 0) continue;
-        int a[4] = {0, 0, 0, 0};
-        a[mu] = d[mu];
+        int a[4] = {mu == 0, mu == 1, mu == 2, mu == 3};
         int rest[4] = {d[0], d[1], d[2], d[3]};
         rest[mu] = 0;
-        const int ca = dir81_of(a), cr = dir81_of(rest);
-        const long sa = s + (d[mu] > 0 ? fwd[mu] : bwd[mu]);
-        cx<double> Va[9], Wr[9];
-        for (int e = 0; e < 9; ++e) {
-            double2 u = tmp[((size_t)ca * 9 + e) * g.vol + s];
-            double2 w = tmp[((size_t)cr * 9 + e) * g.vol + sa];
-            Va[e] = {u.x, u.y};
-            Wr[e] = {w.x, w.y};
-        }
-        for (int r = 0; r < 3; ++r)
-            for (int q = 0; q < 3; ++q) {
-                cx<double> t = acc[r * 3 + q];
-                for (int m = 0; m < 3; ++m) t = cfma(Va[r * 3 + m], Wr[m * 3 + q], t);
-                acc[r * 3 + q] = t;
-            }
+        cx<A> H[9], R[9];
+        load_mat<A>(W, g.vol, P.p[code_of(a)], d[mu] > 0 ? s : s + bwd[mu], d[mu] < 0, H);
+        const int pr = P.p[code_of(rest)];
+        if (pr >= 0) load_mat<A>(W, g.vol, pr, s + (d[mu] > 0 ? fwd[mu] : bwd[mu]), false, R);
+        else load_mat<A>(W, g.vol, -1 - pr, sd, true, R);
+        mm_acc(H, R, acc);
     }
-    const double inv = 1.0 / L.k;
+    const A inv = A(1.0 / L.k);
+#pragma unroll
     for (int e = 0; e < 9; ++e)
-        tmp[((size_t)c * 9 + e) * g.vol + s] = make_double2(acc[e].re * inv, acc[e].im * inv);
+        st_el(W, ((size_t)P.p[c] * 9 + e) * g.vol + s, cx<A>{times(settle(acc[e].re), inv), times(settle(acc[e].im), inv)});
 }
 
-struct RepList {
-    short code[40];
-};
-
-__global__ void k_wbuild_store(Geom g, RepList R, const double2* __restrict__ tmp, double2* W64)
+template <typename A> static cudaError_t build_W_T(const Geom& g, const void* V64, void* W, cudaStream_t st)
 {
-    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;   // (site, rep), site fastest
-    if (i >= g.vol * 40) return;
-    const long s = i % g.vol;
-    const int r = (int)(i / g.vol);
-    for (int e = 0; e < 9; ++e) W64[((size_t)r * 9 + e) * g.vol + s] = tmp[((size_t)R.code[r] * 9 + e) * g.vol + s];
-}
-
-// all 80 directions of W (FP64, [dir81][9][site]; the centre code 40 is not written)
-cudaError_t launch_build_W81(const Geom& g, const void* V64, void* tmp81, cudaStream_t st)
-{
-    double2* tmp = (double2*)tmp81;
-    unsigned nb = (unsigned)((g.vol + 255) / 256);
-    k_wbuild_level1<<<nb, 256, 0, st>>>(g, (const double2*)V64, tmp);
+    const DirPlanes P = dir_planes();
+    const long n1 = g.vol * 36;
+    k_w_level1<A><<<(unsigned)((n1 + 255) / 256), 256, 0, st>>>(g, P, (const double2*)V64, W);
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    for (int k = 2; k <= 4; ++k) {
-        DirList L;
-        L.n = 0;
-        L.k = k;
-        for (int c = 0; c < 81; ++c) {
-            int d[4] = {c % 3 - 1, (c / 3) % 3 - 1, (c / 9) % 3 - 1, (c / 27) % 3 - 1};
-            int kk = (d[0] != 0) + (d[1] != 0) + (d[2] != 0) + (d[3] != 0);
-            if (kk == k) L.code[L.n++] = (short)c;
-        }
+    for (int k = 2; k <= 4 && e == cudaSuccess; ++k) {
+        const DirList L = dirs_of_hops(k, true);
         const long n = g.vol * L.n;
-        k_wbuild_level<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(g, L, tmp);
+        k_w_level<A><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(g, L, P, W);
         e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
     }
-    return cudaSuccess;
+    return e;
 }
 
-cudaError_t launch_build_W(const Geom& g, const void* V64, void* tmp81, void* W64, cudaStream_t st)
+cudaError_t launch_build_W(const Geom& g, const void* V64, void* W, bool df, cudaStream_t st)
 {
-    double2* tmp = (double2*)tmp81;
-    cudaError_t e = launch_build_W81(g, V64, tmp81, st);
-    if (e != cudaSuccess) return e;
-    BriDir dirs[80];
-    int reps[40];
-    brillouin_tables(dirs, reps);
-    RepList R;
-    for (int r = 0; r < 40; ++r) R.code[r] = (short)reps[r];
-    const long n = g.vol * 40;
-    k_wbuild_store<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(g, R, tmp, (double2*)W64);
-    return cudaGetLastError();
+    return df ? build_W_T<dfl>(g, V64, W, st) : build_W_T<double>(g, V64, W, st);
 }
 
 }  // namespace dirac
