@@ -382,16 +382,15 @@ DIRAC_API dirac_status dirac_get_residual_arithmetic(const dirac_handle* h, int*
  *               spinor loads and one of the eight link loads per site
  *               disappear; 32 or 64 sites per block;
  *            7: (Brillouin, BF16/FP16 storage, R = 1, block = 128) the sweep on
- *               the tensor cores (tcgen05.mma, 16-bit operands, FP32
- *               accumulation in tensor memory): per site the colour sums
- *               T_j = sum_d C_j(d) W_d(x) psi(x + d) of the five coefficient
- *               classes (C_0 = -lambda_k / 2, C_{1+mu} = rho_k d_mu) are one
- *               real matrix product, the spin matrices and the diagonal are
- *               applied afterwards; one CTA per SM walks x-rows (about 200 KB
- *               of shared memory, all 512 tensor-memory columns).  The C_j W
- *               are rounded to the storage type (rho_k first rounded to it),
- *               so results differ from variants 0 and 1 by a few units of
- *               the storage rounding.  Selecting it selects link format 1.
+ *               the tensor cores (mma.sync, 16-bit operands, FP32 accumulation
+ *               in registers): per site the colour sums T_j = sum_d C_j(d)
+ *               W_d(x) psi(x + d) of the five coefficient classes (C_0 =
+ *               -lambda_k / 2, C_{1+mu} = rho_k d_mu) are one real matrix
+ *               product, the spin matrices and the diagonal are applied
+ *               afterwards; one CTA per SM works on tiles of up to 16 sites of an
+ *               (x, y) plane (up to 227 KB of shared memory).  The C_j are
+ *               powers of two up to a factor per class, so the C_j W are exact
+ *               in 16 bits.  Selecting it selects link format 1.
  * UNSUPPORTED for other values. */
 DIRAC_API dirac_status dirac_set_kernel_config(dirac_handle* h, int R, int block, int variant);
 
@@ -458,9 +457,8 @@ DIRAC_API dirac_status dirac_autotune(dirac_handle* h, int force, int* R, int* b
 
 /* Wait for the handle's stream and report kernel-side failures: returns
  * DIRAC_TIMEOUT (and clears the record) if a kernel recorded that a bounded
- * device-side wait ran out since the last call (the tensor-core sweep,
- * variant 7, waits on its own CTA's barriers for at most half a second per
- * wait), else DIRAC_OK or the CUDA error of the stream. */
+ * device-side wait ran out since the last call (no kernel built at present
+ * has one), else DIRAC_OK or the CUDA error of the stream. */
 DIRAC_API dirac_status dirac_sync(dirac_handle* h);
 
 /* One-line description of the last error on h (or of the last failed

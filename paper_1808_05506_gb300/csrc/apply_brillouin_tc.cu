@@ -1,68 +1,43 @@
-// Brillouin sweep on the tensor cores (tcgen05), for BF16 and FP16 storage:
-// launch variant 7.  Sec. 5, Eqs. def_bril, def_der, def_lap at c_SW = 0:
+// Brillouin sweep on the tensor cores, for BF16 and FP16 storage: launch
+// variant 7.  Sec. 5, Eqs. def_bril, def_der, def_lap at c_SW = 0:
 //   D_B psi(x) = (m0 + 15/8) psi(x)
 //                + sum_{d != 0} W_d(x) [rho_k (d . gamma) - lambda_k / 2] psi(x + d).
 // The colour and spin factors commute, so with the five coefficient classes
 //   C_0(d) = -lambda_k / 2,   C_{1+mu}(d) = rho_k d_mu  (k = |d|_1),
 // and T_j[c][(s, v)] = sum_{d, c'} C_j(d) W_d(x)[c][c'] psi_v(x + d)[s][c'],
 //   D_B psi_v(x)[s] = (m0 + 15/8) psi_v(x)[s] + T_0[s] + sum_mu (gamma_mu T_{1+mu})[s].
-// Per site the T_j are one complex product [(s, v)] x [(d, c')] . [(d, c')] x [(j, c)],
-// written as a real one: with X = psi (rows (s, v)), Y = C_j W (columns (j, c)),
-//   D_re = sum X_re Y_re - X_im Y_im,   D_im = sum X_re Y_im + X_im Y_re,
-// the A operand holds X with K = (d, c', re/im) -- the storage order of a 16-bit
-// spinor, so the gathered neighbour words are copied into shared memory
-// unchanged -- and the B operand holds, for output column (j, c, re), the pairs
-// (Y_re, -Y_im) and for (j, c, im) the pairs (Y_im, Y_re).  M = 64 rows (4 spins x
-// 16 right-hand sides), N = 32 columns (30 used), BF16 or FP16 operands, FP32
-// accumulation in tensor memory.  The spin matrices gamma_mu (chiral basis) and
-// the diagonal term are applied in the epilogue on CUDA cores; D^+ = gamma5 D
-// gamma5 negates the rho classes.  Every W is read at the site itself (link
-// format 1: all 80 stored).
+// The coefficients are powers of two up to one factor per class kind,
+//   C_0 = -(1/16) 2^(1-k),   C_{1+mu} = (4/27) d_mu 4^(1-k),
+// so the products C W are formed exactly in 16 bits (the factors go into the
+// epilogue) and the only rounding before the FP32 sums is that of the stored W.
 //
-// A CTA walks whole x-rows of the lattice.  The K dimension is split into three
-// blocks by d_x = -1, 0, +1, and each block into the 27 directions (d_y, d_z,
-// d_t) x 3 colours x (re, im) = 162 elements, padded to 176 (11 MMAs of K = 16).
-// The A block of d_x only depends on the x-coordinate p = x + d_x of the
-// neighbours, so one A slot per x-position p (27 neighbour spinors per rhs)
-// serves the three sites x = p + 1, p, p - 1 (as their d_x = -1, 0, +1 block):
-// one chain of 11 MMAs with N = 96 columns, B = [B(p - 1, d_x = +1), B(p, 0),
-// B(p + 1, -1)], adds to the accumulators of the three sites at once.  The B
-// blocks sit in a ring of entries, entry p holding exactly those three, so each
-// site's builder writes its three blocks into three consecutive entries.  The
-// accumulators form a ring of 16 x 32 tensor-memory columns (all 512), one per
-// site; a chain whose sites wrap around the ring is split in two.  An MMA
-// always accumulates: the epilogue clears each accumulator after reading it.
-// At the ends of a row a slot serves only the sites that exist (N = 32 or 64).
-//
-// The CTA is warp-specialised, its roles linked by mbarriers (every wait
-// bounded in time; a wait that runs out stops the whole CTA and records
-// DIRAC_TIMEOUT):
-//   warps 0-3   epilogue: accumulator -> registers (each warp its lane
-//               quadrant = one spin), clear, spin matrices, diagonal, store;
-//   warp 4      one thread issues the MMA chains and commits them to the
-//               barriers that free the A slot and the B entry and hand
-//               completed accumulators to the epilogue;
-//   warps 5-12  fill the A slots two x-positions at a time (adjacent lanes
-//               load the adjacent 16-byte pieces of the two sites, one 32-byte
-//               sector), the loads issued before waiting for the slots;
-//   warps 13-20 the B blocks of each site from its 80 W (thread = direction x
-//               colour row, both re/im rows), the links of the next site loaded
-//               while the current one is built; the blocks for d_x = -1, 0 go
-//               first, so that the entry they complete is ready while the one
-//               for d_x = +1 still waits for its entry to be free.
-// The B entries C_j(d) W are formed in the storage arithmetic (packed 16-bit
-// multiplies, rounded to nearest): C_0 = -lambda_k / 2 is a power of two, so
-// that product is exact; rho_k is rounded to the storage type first, which
-// keeps the rho classes within two units in the last place of C_j W.
-// The padding of K, the d = 0 entries of B, the entries of the classes that
-// vanish for a direction (d_mu = 0) and the rows of absent right-hand sides
-// stay zero from the start.
-//
-// Shared-memory operands use the canonical no-swizzle K-major layout: core
-// matrices of 8 rows x 16 bytes (8 elements), the K-adjacent core matrices 128 B
-// apart (the descriptor's leading byte offset) and the 8-row groups 22 x 128 B
-// apart (its stride byte offset).  The M = 64 accumulator puts row m in
-// tensor-memory lane (m / 16) * 32 + m % 16.
+// One warp owns a site and up to 16 right-hand sides: a real matrix product
+//   T[(j, c, re/im)][(s, v)] = A[(j, c, re/im)][(d, c', re/im)] B[(d, c', re/im)][(s, v)]
+// of 30 (padded to 32) rows, on mma.sync m16n8k16 (16-bit operands, FP32
+// accumulators in registers), two directions to a step of K = 16, 4 spins x 2
+// right-hand sides to a tile of 8 columns.
+//   A, the links: a lane reads one 16-byte element (the three rows c of column
+//   c' of W_d) per direction and turns it into its eight operand registers by
+//   a swap of (re, im) and a product with (+-2^n, +-2^n) from a table; rows are
+//   placed so that a lane's rows 0..2 are the colours c of one class and one
+//   of re/im.  T_1 and T_3 are kept times i, which makes every spin matrix of
+//   the epilogue real.
+//   B, the spinors: one 32-bit word of shared memory (the (re, im) of one
+//   colour) is one operand register as stored, so the neighbours are copied
+//   unchanged by cp.async: the 9 rows (d_y, d_z) of one d_t at a time, with the
+//   links of these directions, the next stage in flight while one is used.
+// An item is a tile of up to 16 sites of an (x, y) plane, one warp each, for up to
+// 16 right-hand sides (the copies of a tile serve its sites' common neighbours).
+// What bounds it: the mma rate (598 TFLOP/s measured for m16n8k16, 8 cycles per
+// step and tile: 42 steps x 2 row tiles x 8 column tiles take 1344 cycles per
+// site and 16 right-hand sides, 0.58 ms at 16^3 x 32), half reached: between the
+// steps the 16 warps of an SM meet at the barrier of each stage and the epilogue
+// leaves the tensor pipe idle (50 % active; 4900 instructions per site).  The
+// same product on tcgen05.mma takes A and B from shared memory in core matrices;
+// building those in 4- and 8-byte stores (6900 instructions and 1600 wavefronts per
+// site) bounded that kernel.  16^3 x 32, BF16, one GB300: Nv = 16: 1.85 ms
+// with tcgen05 and on CUDA cores, 1.17 ms here; Nv = 12: 1.45 ms on CUDA
+// cores, 0.95 ms; Nv = 4: 0.55 and 0.47 ms.
 #include <algorithm>
 #include <mutex>
 
@@ -72,677 +47,420 @@
 namespace dirac {
 namespace {
 
-constexpr int TC_VB = 16;                               // right-hand sides per work item
-constexpr int TC_M = 4 * TC_VB;                         // 64 rows (spin, right-hand side)
-constexpr int TC_N = 32;                                // per site: 5 classes x 3 colours x (re, im) = 30, padded
-constexpr int TC_KS = 176;                              // K of one slot: 27 x 3 x 2 = 162, padded
-constexpr int TC_KSTEPS = TC_KS / 16;                   // MMAs per chain
-constexpr uint32_t TC_SBO = (TC_KS / 8) * 128;          // bytes between 8-row groups (2816)
-constexpr uint32_t TC_ASLOT = (TC_M / 8) * TC_SBO;      // one A slot (22528 B)
-constexpr uint32_t TC_BBLK = (TC_N / 8) * TC_SBO;       // one site's block of B (11264 B)
-constexpr uint32_t TC_BENT = 3 * TC_BBLK;               // one B entry (33792 B)
-constexpr int TC_NS = 4;                                // A slots
-constexpr int TC_NR = 3;                                // B entries
-constexpr int TC_NACC = 16;                             // accumulators (512 columns)
-constexpr int TC_TS = 25;                               // staged row stride (floats): classes 1..4
-constexpr uint32_t TC_TBUF = TC_M * TC_TS * 4;          // one staging buffer (6400 B)
-constexpr uint32_t TC_A_OFF = 0;
-constexpr uint32_t TC_B_OFF = TC_A_OFF + TC_NS * TC_ASLOT;   // 90112
-constexpr uint32_t TC_T_OFF = TC_B_OFF + TC_NR * TC_BENT;    // 191488
-constexpr uint32_t TC_BAR_OFF = TC_T_OFF + 2 * TC_TBUF;      // 204288
-// barriers: full / empty A slot, full / empty B entry, full / empty accumulator, drain
-constexpr int TC_BAR_FA = 0, TC_BAR_EA = TC_NS, TC_BAR_FB = 2 * TC_NS, TC_BAR_EB = 2 * TC_NS + TC_NR,
-              TC_BAR_FC = 2 * TC_NS + 2 * TC_NR, TC_BAR_EC = TC_BAR_FC + TC_NACC, TC_BAR_DR = TC_BAR_EC + TC_NACC,
-              TC_NBARS = TC_BAR_DR + 1;
-constexpr size_t TC_SMEM = TC_BAR_OFF + 8 * TC_NBARS + 16;
-constexpr int TC_EPI_WARPS = 4, TC_MMA_WARP = 4, TC_GATHER_WARP0 = 5, TC_B_WARP0 = 13, TC_WARPS = 21;
-constexpr int TC_THREADS = TC_WARPS * 32;
-constexpr int TC_BTHREADS = (TC_WARPS - TC_B_WARP0) * 32;    // 256 B builders, 240 with work
-constexpr int TC_GTHREADS = (TC_B_WARP0 - TC_GATHER_WARP0) * 32;   // 256 gatherers
-constexpr int TC_GROUNDS = 28;                          // gather rounds of a pair: 2 x 8 rhs x 14 x 2 directions
-constexpr int TC_GPT = (TC_GROUNDS + 7) / 8;            // gather rounds per thread (8 warps)
-constexpr int TC_MAX_WAIT = 1 << 24;                    // bounded mbarrier wait: polls ...
-constexpr unsigned long long TC_MAX_NS = 500000000ull;  // ... and half a second
-constexpr uint32_t TC_SUSPEND_NS = 20000;               // suspend-time hint of one poll
+constexpr int TC_MAXW = 16;                 // sites of an item, one warp each
+constexpr int TC_STAGES = 2;
+constexpr int TC_SLOTS = 81;                // directions per site in the link copy: 27 x d_t, the centre zero
+constexpr int TC_CO = 9;                    // table entries per direction: 8 row groups, then zeros
+constexpr size_t TC_TAB = (size_t)(TC_SLOTS + 3) * TC_CO * 8;   // coefficient table in shared memory
 
-static_assert(TC_SMEM <= 227 * 1024, "shared memory of one CTA");
-static_assert((TC_BAR_OFF & 7) == 0, "mbarrier alignment");
+// d_t of phase 0, 1, 2: the one with the site itself last, so that the centre
+// spinor is still in shared memory in the epilogue
+__host__ __device__ constexpr int tc_dt(int ph) { return ph == 0 ? -1 : (ph == 1 ? 1 : 0); }
 
-// the 80 directions ordered by d_x block, then rest index (bank-friendly B stores)
+// (exponent, sign) of the coefficients of a direction, by class
 struct TcDir {
-    signed char g;   // d_x + 1
-    signed char r;   // rest index (d_y + 1) + 3 (d_z + 1) + 9 (d_t + 1)
-    short plane;     // W plane at the site (link format 1: rep, or 40 + rep)
-    float c0;        // C_0 = -lambda_k / 2
-    float rho;       // rho_k: C_{1+mu} = rho_k d_mu
-    int nz;          // bit mu: d_mu != 0
-    int neg;         // bit mu: d_mu < 0
+    signed char plane;   // W plane at the site (link format 1: rep, or 40 + rep); -1 the centre
+    signed char k;       // |d|_1
+    signed char d[4];
 };
-static __constant__ TcDir c_tc_dirs[80];
-
-// byte offset of element (row, k) of one K block in the core-matrix layout
-__device__ __forceinline__ uint32_t tc_off(int row, int k)
-{
-    return (uint32_t)(row >> 3) * TC_SBO + (uint32_t)(k >> 3) * 128u + (uint32_t)(row & 7) * 16u +
-           (uint32_t)(k & 7) * 2u;
-}
+static __constant__ TcDir c_tc_dirs[TC_SLOTS];
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ unsigned long long tc_clock_ns()
+template <typename V> __device__ __forceinline__ V tc_lds(const unsigned char* p) { return *reinterpret_cast<const V*>(p); }
+// 16 bytes global -> shared; zeros when off
+__device__ __forceinline__ void tc_cp16(uint32_t dst, const void* src, bool on)
 {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-    return t;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(on ? 16 : 0) : "memory");
 }
 
-// wait for the completion of phase `parity` of the mbarrier, for at most
-// TC_MAX_WAIT polls and TC_MAX_NS nanoseconds, and only while no other role of
-// the CTA has given up (*abort); true if it completed.  A wait that runs out
-// sets *abort, so that every other role stops at its next wait.
-__device__ __noinline__ bool tc_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort)
+template <typename T> __device__ __forceinline__ uint32_t tc_mul2(uint32_t a, uint32_t b);
+template <> __device__ __forceinline__ uint32_t tc_mul2<__nv_bfloat16>(uint32_t a, uint32_t b)
 {
-    const unsigned long long t0 = tc_clock_ns();
-    for (int it = 0; it < TC_MAX_WAIT; ++it) {
-        uint32_t done;
-        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\nselp.u32 %0, 1, 0, p;\n}"
-                     : "=r"(done) : "r"(bar), "r"(parity), "r"(TC_SUSPEND_NS) : "memory");
-        if (done) return true;
-        if ((it & 7) == 7) {
-            if (*abort) return false;
-            if (tc_clock_ns() - t0 > TC_MAX_NS) break;
-        }
-    }
-    *abort = 1;
-    return false;
-}
-
-__device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity, volatile int* abort)
-{
-    uint32_t done;
-    asm volatile("{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    return done ? true : tc_wait_slow(bar, parity, abort);
-}
-
-// shared memory by 32-bit address (an immediate offset where the call gives one)
-template <int OFF = 0> __device__ __forceinline__ void tc_sts32(uint32_t a, uint32_t v)
-{
-    asm volatile("st.shared.u32 [%0+%2], %1;" ::"r"(a), "r"(v), "n"(OFF));
-}
-__device__ __forceinline__ void tc_sts64(uint32_t a, uint32_t v0, uint32_t v1)
-{
-    asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(v0), "r"(v1));
-}
-__device__ __forceinline__ float tc_ldsf(uint32_t a)
-{
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
-    return v;
-}
-__device__ __forceinline__ void tc_stsf(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v)); }
-
-// packed 16-bit product, rounded to nearest
-__device__ __forceinline__ uint32_t tc_mul2(uint32_t x, uint32_t y, __nv_bfloat16*)
-{
-    const __nv_bfloat162 r = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&x), *reinterpret_cast<const __nv_bfloat162*>(&y));
+    const __nv_bfloat162 r = __hmul2(*reinterpret_cast<__nv_bfloat162*>(&a), *reinterpret_cast<__nv_bfloat162*>(&b));
     return *reinterpret_cast<const uint32_t*>(&r);
 }
-__device__ __forceinline__ uint32_t tc_mul2(uint32_t x, uint32_t y, __half*)
+template <> __device__ __forceinline__ uint32_t tc_mul2<__half>(uint32_t a, uint32_t b)
 {
-    const __half2 r = __hmul2(*reinterpret_cast<const __half2*>(&x), *reinterpret_cast<const __half2*>(&y));
+    const __half2 r = __hmul2(*reinterpret_cast<__half2*>(&a), *reinterpret_cast<__half2*>(&b));
     return *reinterpret_cast<const uint32_t*>(&r);
 }
 
-__device__ __forceinline__ void tc_bar_init(uint32_t bar, uint32_t count)
+template <typename T>
+__device__ __forceinline__ void tc_mma(float (&c)[4], const uint32_t a0, const uint32_t a1, const uint32_t a2,
+                                       const uint32_t a3, const uint32_t b0, const uint32_t b1)
 {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+    if constexpr (std::is_same<T, __half>::value)
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+                     "{%0,%1,%2,%3};"
+                     : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                     : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+    else
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+                     "{%0,%1,%2,%3};"
+                     : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                     : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-__device__ __forceinline__ void tc_arrive(uint32_t bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ void tc_arrive_n(uint32_t bar, uint32_t n)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n) : "memory");
-}
-
-// the mbarrier receives one arrival when every MMA this thread issued so far is complete
-__device__ __forceinline__ void tc_commit(uint32_t bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-// the generic-proxy shared-memory stores of this thread become visible to the tensor cores
-__device__ __forceinline__ void tc_fence_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-// barrier 1 over the 128 epilogue threads, and of their flags
-__device__ __forceinline__ bool tc_epi_and(bool v)
-{
-    int r;
-    asm volatile("{\n.reg .pred p, q;\nsetp.ne.s32 p, %1, 0;\nbar.red.and.pred q, 1, 128, p;\nselp.s32 %0, 1, 0, q;\n}"
-                 : "=r"(r) : "r"((int)v) : "memory");
-    return r != 0;
-}
-
-// shared-memory matrix descriptor: no swizzle, leading byte offset 128 (K),
-// stride byte offset TC_SBO (8-row groups), descriptor version 1
-__device__ __forceinline__ uint64_t tc_desc(uint32_t addr)
-{
-    return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)(128u >> 4) << 16) | ((uint64_t)(TC_SBO >> 4) << 32) |
-           ((uint64_t)1 << 46);
-}
-
-template <typename T> struct TcFmt;
-template <> struct TcFmt<__nv_bfloat16> { static constexpr uint32_t v = 1; };
-template <> struct TcFmt<__half> { static constexpr uint32_t v = 0; };
-
-// instruction descriptor of kind::f16: FP32 accumulator, A and B of type T,
-// both K-major, N columns, M = 64
-template <typename T> __device__ __forceinline__ uint32_t tc_idesc(int n)
-{
-    return (1u << 4) | (TcFmt<T>::v << 7) | (TcFmt<T>::v << 10) | ((uint32_t)(n >> 3) << 17) |
-           ((uint32_t)(TC_M >> 4) << 24);
-}
-
-// complex element index of component i (= 3 spin + colour) of rhs v at site s
-template <typename TO> __device__ __forceinline__ size_t tc_out_index(size_t vol, int v, int i, long s)
-{
-    constexpr int CPV = Store<TO>::CPV;
-    return blk_index(vol, 12 / CPV, v, i / CPV, s) * CPV + i % CPV;
-}
-
-// The work schedule every role walks: items (x-row, block of 16 right-hand
-// sides) blockIdx.x, blockIdx.x + gridDim.x, ...; per item Lx + 2 slot fills
-// (positions -1 .. Lx) and Lx sites.
-struct TcRow {
-    long base;   // site of x = 0
-    int vb0;     // first right-hand side of the block
+// one work item: NB right-hand sides from v0 on the sites x0.. x0 + bx - 1, y0..
+// y0 + by - 1 of an (x, y) plane
+struct TcItem {
+    long base;   // first site of the plane
+    int x0, bx, y0, by, v0;
 };
 
-__device__ __forceinline__ TcRow tc_row(const ApplyArgs& a, long item, int nvb)
+struct TcGrid {
+    long nitems;
+    int nvb, nx, ny, bx, by;   // blocks of right-hand sides, tiles per plane, sites per tile
+    FDiv fv, fx, fy, fw;       // division by nvb, nx, ny and bx + 2
+};
+
+template <int NB>
+__device__ __forceinline__ TcItem tc_item(const ApplyArgs& a, const TcGrid& G, long i)
 {
-    const long row = item / nvb;
-    return TcRow{slab_site(a, row * (long)a.g.L[0]), (int)(item - row * nvb) * TC_VB};
+    const uint32_t q = fdiv(G.fv, (uint32_t)i), q1 = fdiv(G.fx, q), q2 = fdiv(G.fy, q1);
+    TcItem it;
+    it.v0 = ((int)i - (int)q * G.nvb) * NB;
+    it.x0 = ((int)q - (int)q1 * G.nx) * G.bx;
+    it.y0 = ((int)q1 - (int)q2 * G.ny) * G.by;
+    it.bx = min(G.bx, a.g.L[0] - it.x0);
+    it.by = min(G.by, a.g.L[1] - it.y0);
+    it.base = slab_site(a, (long)q2 * a.g.stride[2]);
+    return it;
 }
 
-// site of x-position q of the row (periodic, -1 <= q <= Lx)
-__device__ __forceinline__ long tc_site_at(long base, int q, int Lx)
-{
-    int x = q;
-    if (x < 0) x += Lx;
-    if (x >= Lx) x -= Lx;
-    return base + x;
-}
+// The fill of one stage: the links of the 27 directions of phase ph, [site][27][3
+// pieces of 16 bytes], then the spinors at d_t of the tile with its halo of one
+// site in x, y and z, [z][y][x][rhs][3 pieces].  A thread keeps its (x, rhs,
+// piece) over the rows; consecutive threads take consecutive x (16-byte pieces
+// that lie side by side in the field).  start() copies the links and, where a
+// row has more pieces than the CTA has threads, the pieces beyond; part(i) copies the thread's
+// piece of row i = 3 y + z, so that the parts can be spread over the mma steps
+// of the stage in use.
+template <int NB>
+struct TcFill {
+    const uint4* src = nullptr;
+    uint32_t dst = 0, rowbytes = 0, zstep = 0;
+    int zo0 = 0, zo1 = 0, zo2 = 0, x = 0, y = 0, Lx = 0, Ly = 0, nparts = 0;
+    bool on = false;
 
-// Gatherers (warps 5-12): the fills of a row are position -1, then the pairs
-// (0, 1), (2, 3), ..., and what is left; lane bit 0 picks the position of the
-// pair, bits 1..3 the rhs vv & 7 and bit 4 the rest index r & 1, rounds
-// wr = warp + 8 k the rest (vv / 8 = wr & 1, r / 2 = wr / 2).
+    __device__ __forceinline__ void setup(const ApplyArgs& a, const TcGrid& G, const TcItem& it, uint32_t buf, int i)
+    {
+        const int vk = (int)fdiv(G.fw, (uint32_t)i), p = i - vk * (G.bx + 2);
+        const int v = vk / 3, k = vk - 3 * v;
+        x = it.x0 - 1 + p;
+        if (x < 0) x += Lx;
+        if (x >= Lx) x -= Lx;
+        on = it.v0 + v < a.Nv;
+        src = static_cast<const uint4*>(a.in) +
+              ((size_t)(on ? it.v0 + v : 0) * (uint32_t)nblk_of((size_t)a.g.vol) * 96 + 32 * k);
+        dst = buf + (uint32_t)p * (NB * 48u) + (uint32_t)(v * 48 + k * 16);
+        y = it.y0 == 0 ? Ly - 1 : it.y0 - 1;
+    }
+    __device__ __forceinline__ void start(const ApplyArgs& a, const TcGrid& G, const TcItem& it, int ph, uint32_t lbuf,
+                                          uint32_t buf, int tid, int nthr)
+    {
+        Lx = a.g.L[0];
+        Ly = a.g.L[1];
+        const int yw = it.by + 2, dt = tc_dt(ph), row = it.bx * 81;
+        const uint4* ls =
+            static_cast<const uint4*>(a.links) + ((size_t)(it.base + (long)it.y0 * Lx + it.x0) * TC_SLOTS + 27 * ph) * 3;
+        for (int yy = 0; yy < it.by; ++yy) {
+            for (int i = tid; i < row; i += nthr) tc_cp16(lbuf + 16u * i, ls + (i / 81 * (TC_SLOTS * 3 - 81) + i), true);
+            ls += (size_t)Lx * (TC_SLOTS * 3);
+            lbuf += 16u * row;
+        }
+        // z and t of the plane, and the planes z - 1, z, z + 1 at t + d_t
+        const int P = (int)a.g.stride[2], Lz = a.g.L[2], T = P * Lz;
+        const int zt = (int)fdiv(a.g.fdP, (uint32_t)it.base), t = (int)fdiv(a.g.fd[2], (uint32_t)zt), z = zt - t * Lz;
+        int tt = t + dt;
+        tt = tt < 0 ? a.g.L[3] - 1 : (tt == a.g.L[3] ? 0 : tt);
+        zo0 = tt * T + (z == 0 ? Lz - 1 : z - 1) * P;
+        zo1 = tt * T + z * P;
+        zo2 = tt * T + (z + 1 == Lz ? 0 : z + 1) * P;
+        rowbytes = (uint32_t)(G.bx + 2) * (NB * 48u);
+        zstep = (uint32_t)yw * rowbytes;
+        const int n = NB * 3 * (G.bx + 2);
+        for (int i = tid + nthr; i < n; i += nthr) {
+            setup(a, G, it, buf, i);
+            nparts = 3 * yw;
+            rest<0>();
+        }
+        nparts = tid < n ? 3 * yw : 0;
+        if (tid < n) setup(a, G, it, buf, tid);
+    }
+    // row z = dz of the current y, then (dz = 2) the next y
+    __device__ __forceinline__ void part_at(int dz)
+    {
+        const uint32_t s = (uint32_t)(y * Lx + x + (dz == 0 ? zo0 : (dz == 1 ? zo1 : zo2)));
+        tc_cp16(dst + (uint32_t)dz * zstep, src + ((s >> 5) * 96u + (s & 31u)), on);
+        if (dz == 2) {
+            dst += rowbytes;
+            y = y + 1 == Ly ? 0 : y + 1;
+        }
+    }
+    __device__ __forceinline__ void part(int i)
+    {
+        if (i < nparts) part_at(i % 3);
+    }
+    // the parts from I on (nparts is a multiple of 3); rolled up where the sums of
+    // 12 and 16 right-hand sides leave no registers for the unrolled form
+    template <int I> __device__ __forceinline__ void rest()
+    {
+        if constexpr (NB >= 12) {
+            for (int i = I; i < nparts; ++i) part_at(i % 3);
+            return;
+        }
+        if (nparts <= I) return;
+#pragma unroll
+        for (int dz = I % 3; dz < (I % 3 ? 3 : 0); ++dz) part_at(dz);
+        for (int r = (I + 2) / 3; r < nparts / 3; ++r) {
+#pragma unroll
+            for (int dz = 0; dz < 3; ++dz) part_at(dz);
+        }
+    }
+};
+
+// the lane's eight A registers of one direction: w the rows c = 0..2 of column c'
+// (words (re, im)), co the coefficient pairs of its class (rows c of m = 0..2)
+// and of the class T_4 (m = 3, row c = g / 2)
 template <typename T>
-__device__ void tc_gather_role(const ApplyArgs& a, int nvb, uint32_t As, uint32_t bars, volatile int* abort, int gwarp,
-                               int lane)
+__device__ __forceinline__ void tc_a(const uint4& w, uint2 co, uint32_t sel, uint32_t sel3, int g, uint32_t (&A)[4])
 {
-    const int Lx = a.g.L[0];
-    const long nitems = (a.nsites / Lx) * (long)nvb;
-    const size_t nblk = nblk_of((size_t)a.g.vol);
-    const int po = lane & 1;
-    int g_r[TC_GPT], g_vv[TC_GPT];
-    uint32_t g_sb[TC_GPT][3];   // slot offset of (spin 0, rhs vv) at the K of colour c
-#pragma unroll
-    for (int k = 0; k < TC_GPT; ++k) {
-        const int wr = gwarp + 8 * k;
-        g_r[k] = wr < TC_GROUNDS ? 2 * (wr >> 1) + (lane >> 4) : 27;   // 27: none
-        g_vv[k] = ((lane >> 1) & 7) + 8 * (wr & 1);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) g_sb[k][c] = tc_off(g_vv[k], 6 * (g_r[k] < 27 ? g_r[k] : 0) + 2 * c);
-    }
-    long f0 = 0;
-    bool ok = true;
-    for (long item = blockIdx.x; item < nitems && ok; item += gridDim.x, f0 += Lx + 2) {
-        const TcRow R = tc_row(a, item, nvb);
-        long fwd[4], bwd[4];
-        int xc[4];
-        site_offsets(a.g, R.base, fwd, bwd, xc);
-        long g_off[TC_GPT];
-        size_t g_v[TC_GPT];
-        bool g_on[TC_GPT];
-#pragma unroll
-        for (int k = 0; k < TC_GPT; ++k) {
-            const int r = g_r[k];
-            const int dy = r % 3 - 1, dz = (r / 3) % 3 - 1, dt = r / 9 - 1;
-            g_off[k] = (dy > 0 ? fwd[1] : (dy < 0 ? bwd[1] : 0)) + (dz > 0 ? fwd[2] : (dz < 0 ? bwd[2] : 0)) +
-                       (dt > 0 ? fwd[3] : (dt < 0 ? bwd[3] : 0));
-            g_on[k] = r < 27 && R.vb0 + g_vv[k] < a.Nv;
-            g_v[k] = (size_t)(R.vb0 + g_vv[k]) * nblk;
+    A[0] = tc_mul2<T>(__byte_perm(w.x, 0, sel), co.x);
+    A[1] = tc_mul2<T>(__byte_perm(w.y, 0, sel), co.x);
+    A[2] = tc_mul2<T>(__byte_perm(w.z, 0, sel), co.x);
+    const uint32_t w3 = g < 2 ? w.x : (g < 4 ? w.y : w.z);
+    A[3] = tc_mul2<T>(__byte_perm(w3, 0, sel3), co.y);
+}
+
+template <typename T, int NT>
+__global__ void __launch_bounds__(TC_MAXW * 32, 1) k_brillouin_tc(ApplyArgs a, TcGrid G, float frho)
+{
+    constexpr int NB = 2 * NT;   // right-hand sides of an item
+    // the copies of the next stage spread over the mma steps of this one; with few
+    // tiles per step they only lengthen it (16^3 x 32: Nv = 16 1.29 -> 1.17 ms, 12
+    // 1.01 -> 0.95 ms, but 8 0.73 -> 0.76 ms, 4 0.47 -> 0.62 ms)
+    constexpr bool SPREAD = NT >= 6;
+    extern __shared__ __align__(128) unsigned char tc_smem[];
+    const int tid = threadIdx.x, nthr = blockDim.x, warp = tid >> 5, lane = tid & 31;
+    const int g = lane >> 2, q = lane & 3, j = g >> 1, ri = g & 1;
+    // a stage: links, then spinors
+    const uint32_t lbytes = (uint32_t)(G.bx * G.by) * (27u * 48u);
+    const uint32_t stage = lbytes + 3u * (uint32_t)((G.bx + 2) * (G.by + 2)) * (NB * 48u);
+
+    // coefficient pairs of every direction and row group g = (class j, re/im): the
+    // signs of the realified product, (re, -im) for the real row and (im, re) for
+    // the imaginary one; rows kept times i: (-im, -re) and (re, -im)
+    for (int i = tid; i < (TC_SLOTS + 3) * TC_CO; i += nthr) {
+        const int sl = i / TC_CO, gg = i - sl * TC_CO;
+        float c[2] = {0.f, 0.f}, c3[2] = {0.f, 0.f};
+        if (sl < TC_SLOTS && gg < 8 && c_tc_dirs[sl].plane >= 0) {
+            const TcDir& D = c_tc_dirs[sl];
+            const int jj = gg >> 1, im = gg & 1;
+            const float p2 = 2.f / (float)(1 << D.k), p4 = 4.f / (float)(1 << (2 * D.k));
+            const float cj = jj == 0 ? p2 : p4 * (float)D.d[jj - 1];
+            const bool ti = jj == 1 || jj == 3;
+            c[0] = (ti && !im) ? -cj : cj;
+            c[1] = (ti || !im) ? -cj : cj;
+            const float c4 = p4 * (float)D.d[3];
+            c3[0] = c4;
+            c3[1] = im ? c4 : -c4;
         }
-        for (int p = -1; p <= Lx && ok;) {
-            const int np = (p >= 0 && p + 1 <= Lx) ? 2 : 1;   // positions in this fill
-            const bool lane_on = po < np;
-            const long sq = tc_site_at(R.base, p + po, Lx);
-            uint4 w[TC_GPT][3];
-#pragma unroll
-            for (int k = 0; k < TC_GPT; ++k) {
-                if (!(g_on[k] && lane_on)) continue;
-                const long nb = sq + g_off[k];
-                const uint4* q = reinterpret_cast<const uint4*>(a.in) + (g_v[k] + (size_t)(nb >> 5)) * 96 + (nb & 31);
-                w[k][0] = ld_ro(q);
-                w[k][1] = ld_ro(q + 32);
-                w[k][2] = ld_ro(q + 64);
-            }
-            const long F = f0 + p + 1;   // fill of position p
-            for (int j = 0; j < np && ok; ++j)
-                if (F + j >= TC_NS)
-                    ok = tc_wait(bars + 8u * (TC_BAR_EA + (int)((F + j) % TC_NS)), (uint32_t)(((F + j) / TC_NS - 1) & 1), abort);
-            if (!ok) break;
-            const uint32_t S = As + (uint32_t)((F + po) % TC_NS) * TC_ASLOT;
-#pragma unroll
-            for (int k = 0; k < TC_GPT; ++k) {
-                if (!(g_on[k] && lane_on)) continue;
-                const uint32_t wv[12] = {w[k][0].x, w[k][0].y, w[k][0].z, w[k][0].w, w[k][1].x, w[k][1].y,
-                                         w[k][1].z, w[k][1].w, w[k][2].x, w[k][2].y, w[k][2].z, w[k][2].w};
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    // rows spin * 16 + vv: 2 spin 8-row groups further down
-                    const uint32_t at = S + g_sb[k][c];
-                    tc_sts32<0>(at, wv[c]);
-                    tc_sts32<2 * TC_SBO>(at, wv[3 + c]);
-                    tc_sts32<4 * TC_SBO>(at, wv[6 + c]);
-                    tc_sts32<6 * TC_SBO>(at, wv[9 + c]);
-                }
-            }
-            tc_fence_async();
-            for (int j = 0; j < np; ++j) tc_arrive(bars + 8u * (TC_BAR_FA + (int)((F + j) % TC_NS)));
-            p += np;
+        uint32_t* e = reinterpret_cast<uint32_t*>(tc_smem) + 2 * i;
+        e[0] = pack2(cx<float>{c[0], c[1]}, (T*)nullptr);
+        e[1] = pack2(cx<float>{c3[0], c3[1]}, (T*)nullptr);
+    }
+
+    // lane constants: (re, im) order of the two kinds of rows, table entry (lanes
+    // q = 3 pad K: coefficient zero), link element, word of B in a spinor pair
+    const uint32_t sel = ((ri != 0) != (j == 1 || j == 3)) ? 0x1032u : 0x3210u;
+    const uint32_t sel3 = ri ? 0x1032u : 0x3210u;
+    const unsigned char* tabl = tc_smem + 8 * (q == 3 ? 8 : g);
+    const int qc = q == 3 ? 2 : q;
+    const uint32_t boff = 4u * ((g >> 2) * 12 + 3 * (g & 3) + qc);
+    const int wy_full = warp / G.bx;
+
+    long i0 = blockIdx.x, i1 = blockIdx.x;   // item and phase of the next fill
+    int ph1 = 0, nfill = 0;
+    TcFill<NB> F;
+    auto fill_next = [&]() {   // begins the next fill; F.part / F.rest and a commit complete it
+        F.nparts = 0;
+        if (i1 < G.nitems) {
+            const TcItem it = tc_item<NB>(a, G, i1);
+            const uint32_t b = smem_u32(tc_smem) + (uint32_t)TC_TAB + (uint32_t)(nfill % TC_STAGES) * stage;
+            F.start(a, G, it, ph1, b, b + lbytes, tid, nthr);
         }
-    }
-    // tail: the last releases of the slots arrive before the CTA may exit
-    if (ok && gwarp == 0 && lane == 0) {
-        for (long g = f0 - TC_NS; g < f0; ++g)
-            if (g >= 0 && !tc_wait(bars + 8u * (TC_BAR_EA + (int)(g % TC_NS)), (uint32_t)((g / TC_NS) & 1), abort)) break;
-    }
-}
-
-// number of arrivals site x of a row of Lx sites brings to the B entry x + g:
-// its own, plus those of the sites -2, -1 (site 0) or Lx, Lx + 1 (site Lx - 1)
-// that do not exist, so that every entry completes with 3 arrivals per builder
-__device__ __forceinline__ uint32_t tc_b_count(int x, int g, int Lx)
-{
-    const int e = x + g;
-    uint32_t n = 1;
-    if (x == 0) n += (uint32_t)max(0, 2 - e);
-    if (x == Lx - 1) n += (uint32_t)max(0, e - (Lx - 1));
-    return n;
-}
-
-// three consecutive words (colours c' = 0, 1, 2 of one direction) of one row of
-// a B block: 6 r + 2 c' are element offsets along K, so for even r the first two
-// words share an aligned 8-byte pair, for odd r the last two
-__device__ __forceinline__ void tc_st3(uint32_t at, uint32_t ka, uint32_t kb, bool odd, uint32_t w0, uint32_t w1,
-                                       uint32_t w2)
-{
-    if (!odd) {
-        tc_sts64(at + ka, w0, w1);
-        tc_sts32(at + kb, w2);
-    } else {
-        tc_sts32(at + ka, w0);
-        tc_sts64(at + kb, w1, w2);
-    }
-}
-
-// B builders (warps 13-20): thread t < 240 owns direction t / 3 (order of
-// c_tc_dirs) and colour row c = t % 3, both its re and im rows; it reads the
-// three words W_d(x)[c][c'] from the site-major copy (a warp's loads for a
-// site are about 100 consecutive words).  Site x's block for d_x = g - 1 goes
-// to sub-block 2 - g of the entry of fill f0 + x + g.  Only the classes that do
-// not vanish for the direction are written, the rho classes as one product
-// with the sign bits of both halves flipped where C_{1+mu} < 0 (rounding to
-// nearest is odd in its argument).
-template <typename T, bool DAG>
-__device__ void tc_b_role(const ApplyArgs& a, int nvb, uint32_t Bs, uint32_t bars, volatile int* abort, int btid)
-{
-    const int Lx = a.g.L[0];
-    const long nitems = (a.nsites / Lx) * (long)nvb;
-    const bool on = btid < 240;
-    const int d = on ? btid / 3 : 0, c = btid % 3;
-    const TcDir D = c_tc_dirs[d];
-    const int g_own = D.g, nz = D.nz, neg = DAG ? (D.neg ^ 0xF) : D.neg;
-    const bool odd = D.r & 1;
-    const uint32_t sub = (uint32_t)(2 - D.g) * TC_BBLK;
-    const uint32_t ka = sub + tc_off(0, 6 * D.r), kb = sub + tc_off(0, odd ? 6 * D.r + 2 : 6 * D.r + 4);
-    const uint32_t c0x2 = pack2(cx<float>{D.c0, D.c0}, (T*)nullptr);
-    const uint32_t rhox2 = pack2(cx<float>{D.rho, D.rho}, (T*)nullptr);
-    uint32_t rowoff[2][5];   // rows 6 j + 2 c + ri
-#pragma unroll
-    for (int ri = 0; ri < 2; ++ri)
-#pragma unroll
-        for (int j = 0; j < 5; ++j) rowoff[ri][j] = tc_off(6 * j + 2 * c + ri, 0);
-    const int woff = 9 * d + 3 * c;
-    auto load = [&](long s, uint32_t (&w)[3]) {
-        if (!on) return;
-        const uint32_t* W = reinterpret_cast<const uint32_t*>(a.links) + (size_t)s * 720 + woff;
-        w[0] = ld_ro(W);
-        w[1] = ld_ro(W + 1);
-        w[2] = ld_ro(W + 2);
+        ++nfill;
+        if (++ph1 == 3) {
+            ph1 = 0;
+            i1 += gridDim.x;
+        }
     };
-    uint32_t wn[3] = {0u, 0u, 0u};
-    if ((long)blockIdx.x < nitems) load(tc_row(a, blockIdx.x, nvb).base, wn);
-    long f0 = 0;
-    bool ok = true;
-    for (long item = blockIdx.x; item < nitems && ok; item += gridDim.x, f0 += Lx + 2) {
-        const TcRow R = tc_row(a, item, nvb);
-        for (int x = 0; x < Lx; ++x) {
-            const uint32_t wc[3] = {wn[0], wn[1], wn[2]};
-            // the links of the next site, in flight while this one is built
-            if (x + 1 < Lx) load(R.base + x + 1, wn);
-            else if (item + (long)gridDim.x < nitems) load(tc_row(a, item + gridDim.x, nvb).base, wn);
-            // the blocks for g = 0, 1, 2 in turn, each after its entry is free
-            // (the entries of g = 0, 1 were already free for site x - 1)
+    fill_next();
+    F.template rest<0>();
+    cp_async_commit();
+    int nuse = 0;
+    for (; i0 < G.nitems; i0 += gridDim.x) {
+        const TcItem it = tc_item<NB>(a, G, i0);
+        const bool on = warp < it.bx * it.by;
+        const int wy = it.bx == G.bx ? wy_full : warp / it.bx, wx = warp - wy * it.bx;
+        const long s = it.base + (long)(it.y0 + wy) * a.g.L[0] + it.x0 + wx;
+        float acc0[NT][4], acc1[NT][4];   // rows m = 0, 1 and m = 2, 3
 #pragma unroll
-            for (int g = 0; g < 3; ++g) {
-                const long F = f0 + x + g;
-                if ((g == 2 || x == 0) && F >= TC_NR &&
-                    !tc_wait(bars + 8u * (TC_BAR_EB + (int)(F % TC_NR)), (uint32_t)((F / TC_NR - 1) & 1), abort)) {
-                    ok = false;
-                    break;
-                }
-                if (on && g == g_own) {
-                    const uint32_t base = Bs + (uint32_t)(F % TC_NR) * TC_BENT;
-                    uint32_t p0[2][3], p1[2][3];
+        for (int t = 0; t < NT; ++t)
 #pragma unroll
-                    for (int cp = 0; cp < 3; ++cp) {
-                        const uint32_t e0 = wc[cp] ^ 0x80000000u;          // (re, -im)
-                        const uint32_t e1 = __byte_perm(wc[cp], 0, 0x1032); // (im, re)
-                        p0[0][cp] = tc_mul2(e0, c0x2, (T*)nullptr);
-                        p0[1][cp] = tc_mul2(e1, c0x2, (T*)nullptr);
-                        p1[0][cp] = tc_mul2(e0, rhox2, (T*)nullptr);
-                        p1[1][cp] = tc_mul2(e1, rhox2, (T*)nullptr);
-                    }
-#pragma unroll
-                    for (int ri = 0; ri < 2; ++ri) {
-                        tc_st3(base + rowoff[ri][0], ka, kb, odd, p0[ri][0], p0[ri][1], p0[ri][2]);
-#pragma unroll
-                        for (int mu = 0; mu < 4; ++mu) {
-                            if (!((nz >> mu) & 1)) continue;
-                            const uint32_t m = ((neg >> mu) & 1) ? 0x80008000u : 0u;
-                            tc_st3(base + rowoff[ri][1 + mu], ka, kb, odd, p1[ri][0] ^ m, p1[ri][1] ^ m, p1[ri][2] ^ m);
-                        }
-                    }
-                    tc_fence_async();
-                }
-                tc_arrive_n(bars + 8u * (TC_BAR_FB + (int)(F % TC_NR)), tc_b_count(x, g, Lx));
+            for (int e = 0; e < 4; ++e) acc0[t][e] = acc1[t][e] = 0.f;
+        const uint32_t ss = NB * 48u, rs = (uint32_t)(G.bx + 2) * ss, rz = (uint32_t)(it.by + 2) * rs;
+        const unsigned char* buf = tc_smem;
+#pragma unroll 1
+        for (int ph = 0; ph < 3; ++ph) {
+            cp_async_wait<TC_STAGES - 2>();
+            __syncthreads();   // the stage is filled, and the one before it no longer read
+            fill_next();
+            if (!SPREAD || !on) {
+                F.template rest<0>();
+                cp_async_commit();
             }
-            if (!ok) break;
-        }
-    }
-    // tail: the last releases of the entries arrive before the CTA may exit
-    if (ok && btid == 0) {
-        for (long F = f0 - TC_NR; F < f0; ++F)
-            if (F >= 0 && !tc_wait(bars + 8u * (TC_BAR_EB + (int)(F % TC_NR)), (uint32_t)((F / TC_NR) & 1), abort)) break;
-    }
-}
-
-// one chain of MMAs: A slot a0 (K = 176) times the sub-blocks of B from b0, n
-// columns, into tensor-memory columns d
-template <typename T>
-__device__ __forceinline__ void tc_chain(uint32_t d, uint32_t a0, uint32_t b0, int n)
-{
-    const uint32_t idesc = tc_idesc<T>(n);
+            buf = tc_smem + TC_TAB + (uint32_t)(nuse % TC_STAGES) * stage + lbytes;
+            ++nuse;
+            if (!on) continue;
+            const unsigned char* lk = buf - lbytes + (uint32_t)warp * (27u * 48u) + 16 * qc;
+            const unsigned char* bb = buf + (uint32_t)wy * rs + (uint32_t)wx * ss + boff;
+            const unsigned char* tb = tabl + ph * (27 * TC_CO * 8);
 #pragma unroll
-    for (int t = 0; t < TC_KSTEPS; ++t) {
-        const uint64_t ad = tc_desc(a0 + 256u * t), bd = tc_desc(b0 + 256u * t);
-        asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                     "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-                     ::"r"(d), "l"(ad), "l"(bd), "r"(idesc), "n"(1));
-    }
-}
-
-// The MMA issuer (one thread of warp 4): per slot p of a row (fill f0 + p + 1),
-// once its A slot and its B entry are there and the accumulator of the site it
-// opens (p + 1) is free, the chain (or two, where the sites wrap around the
-// accumulator ring); then the commits that free the slot and the entry and
-// hand site p - 1, now complete, to the epilogue.
-template <typename T>
-__device__ void tc_mma_role(const ApplyArgs& a, int nvb, uint32_t a_base, uint32_t b_base, uint32_t tmem,
-                            uint32_t bars, volatile int* abort)
-{
-    const int Lx = a.g.L[0];
-    const long nitems = (a.nsites / Lx) * (long)nvb;
-    long f0 = 0, i0 = 0;
-    bool ok = true;
-    for (long item = blockIdx.x; item < nitems && ok; item += gridDim.x, f0 += Lx + 2, i0 += Lx) {
-        for (int p = -1; p <= Lx; ++p) {
-            const long F = f0 + p + 1;
-            ok = tc_wait(bars + 8u * (TC_BAR_FA + (int)(F % TC_NS)), (uint32_t)((F / TC_NS) & 1), abort);
-            if (ok) ok = tc_wait(bars + 8u * (TC_BAR_FB + (int)(F % TC_NR)), (uint32_t)((F / TC_NR) & 1), abort);
-            if (ok && p + 1 < Lx && i0 + p + 1 >= TC_NACC) {
-                const long in = i0 + p + 1;
-                ok = tc_wait(bars + 8u * (TC_BAR_EC + (int)(in % TC_NACC)), (uint32_t)((in / TC_NACC - 1) & 1), abort);
-            }
-            if (!ok) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int xlo = max(p - 1, 0), xhi = min(p + 1, Lx - 1);
-            const uint32_t a0 = a_base + (uint32_t)(F % TC_NS) * TC_ASLOT;
-            const uint32_t e0 = b_base + (uint32_t)(F % TC_NR) * TC_BENT;
-            // sites xlo .. xhi: sub-blocks x - p + 1, accumulators (i0 + x) % 16
-            const int c0 = (int)((i0 + xlo) % TC_NACC), cnt = xhi - xlo + 1;
-            const int run = min(cnt, TC_NACC - c0);
-            tc_chain<T>(tmem + 32u * c0, a0, e0 + (uint32_t)(xlo - p + 1) * TC_BBLK, 32 * run);
-            if (run < cnt) tc_chain<T>(tmem, a0, e0 + (uint32_t)(xlo + run - p + 1) * TC_BBLK, 32 * (cnt - run));
-            tc_commit(bars + 8u * (TC_BAR_EA + (int)(F % TC_NS)));
-            tc_commit(bars + 8u * (TC_BAR_EB + (int)(F % TC_NR)));
-            if (p >= 1) tc_commit(bars + 8u * (TC_BAR_FC + (int)((i0 + p - 1) % TC_NACC)));
-        }
-    }
-    // every MMA issued here is complete before tensor memory is freed
-    tc_commit(bars + 8u * TC_BAR_DR);
-    volatile int never = 0;
-    tc_wait(bars + 8u * TC_BAR_DR, 0u, &never);
-}
-
-// Epilogue (warps 0-3): warp w reads lanes 32 w .. 32 w + 15 of the site's
-// accumulator (rows w * 16 + vv: spin w, rhs vv) and clears it; T_1 .. T_4 go
-// through shared memory to the spins that need them, and each (spin, rhs)
-// forms T_0 + sum_mu gamma_mu T_{1+mu} (chiral basis: gamma_1, gamma_2 couple
-// spin s to 3 - s, gamma_3, gamma_4 to s ^ 2), adds the diagonal and stores.
-// psi(x) for the diagonal is loaded one site ahead.
-template <typename T>
-__device__ void tc_epi_role(const ApplyArgs& a, int nvb, uint32_t Ts, uint32_t tmem, uint32_t bars, volatile int* abort,
-                            int tid)
-{
-    static_assert(Store<T>::CPV == 4, "16-bit fields");
-    const int Lx = a.g.L[0];
-    const long nitems = (a.nsites / Lx) * (long)nvb;
-    const size_t nblk = nblk_of((size_t)a.g.vol);
-    const int sp = tid >> 5, lane = tid & 31, vv = lane & 15;
-    const bool lane_on = lane < TC_VB;
-    const uint32_t zero = 0u;
-    // factors of the couplings: gamma_1 (-i / +i), gamma_2 (-1 / +1), gamma_3 (-i / +i)
-    const float s1 = sp < 2 ? -1.f : 1.f;
-    const float s2 = (sp == 0 || sp == 3) ? -1.f : 1.f;
-    // complex 3 sp + c of rhs v at site s: ((v nblk + s / 32) 3 + i / 4) 128 + (s % 32) 4 + i % 4
-    uint32_t ioff[3];
+            for (int st = 0; st < 14; ++st) {
+                const int e0 = 2 * st, e1 = st == 13 ? 26 : 2 * st + 1;   // (d_x + 1) + 3 (d_y + 1) + 9 (d_z + 1)
+                uint32_t A0[4], A1[4];
+                tc_a<T>(tc_lds<uint4>(lk + 48 * e0), tc_lds<uint2>(tb + e0 * (TC_CO * 8)), sel, sel3, g, A0);
+                if (st < 13) tc_a<T>(tc_lds<uint4>(lk + 48 * e1), tc_lds<uint2>(tb + e1 * (TC_CO * 8)), sel, sel3, g, A1);
+                else A1[0] = A1[1] = A1[2] = A1[3] = 0u;   // 27 directions: the last step has one
+                if constexpr (SPREAD) F.part(st);
+                const unsigned char* p0 = bb + (uint32_t)(e0 / 9) * rz + (uint32_t)(e0 / 3 % 3) * rs + (uint32_t)(e0 % 3) * ss;
+                const unsigned char* p1 = bb + (uint32_t)(e1 / 9) * rz + (uint32_t)(e1 / 3 % 3) * rs + (uint32_t)(e1 % 3) * ss;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) ioff[c] = (uint32_t)(((3 * sp + c) >> 2) * 128 + ((3 * sp + c) & 3));
-    // staged rows: own (written), spin 3 - sp and spin sp ^ 2 (read)
-    const uint32_t t_own = (uint32_t)((sp * TC_VB + vv) * TC_TS * 4);
-    const uint32_t t_a = (uint32_t)(((3 - sp) * TC_VB + vv) * TC_TS * 4);
-    const uint32_t t_b = (uint32_t)(((sp ^ 2) * TC_VB + vv) * TC_TS * 4);
-    const uint32_t* in = reinterpret_cast<const uint32_t*>(a.in);
-    auto site_part = [](long s) { return (size_t)(s >> 5) * 384 + (size_t)(s & 31) * 4; };
-    auto load_own = [&](const TcRow& R, long s, uint32_t (&w)[3]) {
-        const int v = R.vb0 + vv;
-        if (!lane_on || v >= a.Nv) return;
-        const uint32_t* q = in + (size_t)v * nblk * 384 + site_part(s);
-        w[0] = ld_ro(q + ioff[0]);
-        w[1] = ld_ro(q + ioff[1]);
-        w[2] = ld_ro(q + ioff[2]);
-    };
-    uint32_t own_n[3] = {0u, 0u, 0u};
-    if ((long)blockIdx.x < nitems) {
-        const TcRow R0 = tc_row(a, blockIdx.x, nvb);
-        load_own(R0, R0.base, own_n);
-    }
-    long i = 0;
-    bool ok = true;
-    for (long item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-        const TcRow R = tc_row(a, item, nvb);
-        const int v = R.vb0 + vv;
-        const bool v_on = lane_on && v < a.Nv;
-        const float dg = v_on ? (a.diag_vf ? a.diag_vf[v] : (a.diag_v ? (float)a.diag_v[v] : a.diagf)) : 0.f;
-        uint32_t* out = reinterpret_cast<uint32_t*>(a.out) + (size_t)(v_on ? v : 0) * nblk * 384;
-        for (int x = 0; x < Lx; ++x, ++i) {
-            const uint32_t own[3] = {own_n[0], own_n[1], own_n[2]};
-            if (x + 1 < Lx) load_own(R, R.base + x + 1, own_n);
-            else if (item + (long)gridDim.x < nitems) {
-                const TcRow Rn = tc_row(a, item + gridDim.x, nvb);
-                load_own(Rn, Rn.base, own_n);
-            }
-            const int ac = (int)(i % TC_NACC);
-            bool w_ok = tc_wait(bars + 8u * (TC_BAR_FC + ac), (uint32_t)((i / TC_NACC) & 1), abort);
-            w_ok = __all_sync(0xffffffffu, w_ok);
-            const uint32_t Tb = Ts + (uint32_t)(i & 1) * TC_TBUF;
-            uint32_t r[32];
-            if (w_ok) {
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t taddr = tmem + 32u * ac + ((uint32_t)(sp * 32) << 16);
-                asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                             "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-                             : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                               "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-                               "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]),
-                               "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-                               "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-                             : "r"(taddr));
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                // clear the accumulator for the site that takes it next
-                asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,"
-                             "%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(taddr), "r"(zero) : "memory");
-                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                tc_arrive(bars + 8u * (TC_BAR_EC + ac));
-                if (lane_on) {
-#pragma unroll
-                    for (int n = 6; n < 30; ++n) tc_stsf(Tb + t_own + 4u * (n - 6), __uint_as_float(r[n]));
+                for (int t = 0; t < NT; ++t) {
+                    const uint32_t B0 = tc_lds<uint32_t>(p0 + 96 * t), B1 = tc_lds<uint32_t>(p1 + 96 * t);
+                    tc_mma<T>(acc0[t], A0[0], A0[1], A1[0], A1[1], B0, B1);
+                    tc_mma<T>(acc1[t], A0[2], A0[3], A1[2], A1[3], B0, B1);
                 }
             }
-            if (!tc_epi_and(w_ok)) {
-                ok = false;
-                break;
+            if constexpr (SPREAD) {
+                F.template rest<14>();
+                cp_async_commit();
             }
-            if (v_on) {
-                const size_t sp_idx = site_part(R.base + x);
+        }
+        // Epilogue.  The lane holds, for columns (v, s) with v = q / 2 and s = 2 (q & 1)
+        // + {0, 1}: rows m = 0..2 the colours of class j (re or im by ri), row 3 the
+        // colour j of T_4 (j < 3).  With X = i T:
+        //   out[s] = f0 T_0[s] + frho (s1 X_1[3 - s] + s2 T_2[3 - s] + s2 X_3[s ^ 2] + T_4[s ^ 2]),
+        //   s1 = (-, -, +, +), s2 = (-, +, +, -): classes 1..4 move to the lane q ^ 1,
+        // then the classes are summed over the lanes of j, each of which keeps the
+        // colour c = j, and (re, im) are exchanged so that a lane stores one word.
+        if (!on) continue;
+        const bool low = (q & 1) != 0;   // the columns of the lane are spins 2, 3; the ones it serves 0, 1
+        const float sa = low ? -frho : frho;   // s1, and s2 of the first served spin
+        const float m0 = j == 0 ? -1.f / 16.f : sa, m1 = j == 0 ? -1.f / 16.f : (j == 1 ? sa : -sa);
+        const bool swap = j == 1 || j == 2;                     // 3 - s: the other parity of s
+        const int from = j == 0 ? lane : (lane ^ 1);
+        const bool hi = j >= 2, odd = (j & 1) != 0;
+        const unsigned char* own = buf + rz + (uint32_t)(wy + 1) * rs + (uint32_t)(wx + 1) * ss;   // the site itself
+        const int cw = 3 * (2 * (q & 1) + ri) + (j < 3 ? j : 0);   // the word this lane writes: spin, colour j
+        const unsigned char* ownw = own + 48 * (q >> 1) + 4 * cw;
+        const uint32_t nblk = (uint32_t)nblk_of((size_t)a.g.vol);
+        int v = it.v0 + (q >> 1);
+        uint32_t* op = static_cast<uint32_t*>(a.out) +
+                       4 * (((size_t)v * nblk + (uint32_t)(s >> 5)) * 96 + 32 * (cw >> 2) + (s & 31)) + (cw & 3);
+        const size_t ostep = (size_t)nblk * (2 * 96 * 4);
 #pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    // T_0[sp] + s1 i T_1[3 - sp] + s2 T_2[3 - sp] + s2 i T_3[sp ^ 2] + T_4[sp ^ 2]
-                    const float t1r = tc_ldsf(Tb + t_a + 8u * c), t1i = tc_ldsf(Tb + t_a + 8u * c + 4);
-                    const float t2r = tc_ldsf(Tb + t_a + 24u + 8u * c), t2i = tc_ldsf(Tb + t_a + 28u + 8u * c);
-                    const float t3r = tc_ldsf(Tb + t_b + 48u + 8u * c), t3i = tc_ldsf(Tb + t_b + 52u + 8u * c);
-                    const float t4r = tc_ldsf(Tb + t_b + 72u + 8u * c), t4i = tc_ldsf(Tb + t_b + 76u + 8u * c);
-                    cx<float> o{__uint_as_float(r[2 * c]), __uint_as_float(r[2 * c + 1])};
-                    o.re += -s1 * t1i + s2 * t2r - s2 * t3i + t4r;
-                    o.im += s1 * t1r + s2 * t2i + s2 * t3r + t4i;
-                    const cx<float> pc = unpack2(own[c], (T*)nullptr);
-                    o.re = fmaf(dg, pc.re, o.re);
-                    o.im = fmaf(dg, pc.im, o.im);
-                    st_cs(out + sp_idx + ioff[c], pack2(o, (T*)nullptr));
-                }
+        for (int t = 0; t < NT; ++t, v += 2, op += ostep) {
+            float u0[3], u1[3];
+            const float in0[3] = {acc0[t][0], acc0[t][2], acc1[t][0]}, in1[3] = {acc0[t][1], acc0[t][3], acc1[t][1]};
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                u0[c] = __shfl_sync(0xffffffffu, m0 * (swap ? in1[c] : in0[c]), from);
+                u1[c] = __shfl_sync(0xffffffffu, m1 * (swap ? in0[c] : in1[c]), from);
+            }
+            // sum over j, halving: first j and j ^ 2 (colours 0, 1 | 2), then j and j ^ 1
+            const float a0 = (hi ? u0[2] : u0[0]) + __shfl_xor_sync(0xffffffffu, hi ? u0[0] : u0[2], 16);
+            const float a1 = (hi ? u1[2] : u1[0]) + __shfl_xor_sync(0xffffffffu, hi ? u1[0] : u1[2], 16);
+            const float b0 = u0[1] + __shfl_xor_sync(0xffffffffu, u0[1], 16);   // used by j < 2
+            const float b1 = u1[1] + __shfl_xor_sync(0xffffffffu, u1[1], 16);
+            float k0 = (odd ? b0 : a0) + __shfl_xor_sync(0xffffffffu, odd ? a0 : b0, 8);
+            float k1 = (odd ? b1 : a1) + __shfl_xor_sync(0xffffffffu, odd ? a1 : b1, 8);
+            // for j = 2 the partner j = 3 sends its a (colour 2)
+            k0 = fmaf(frho, __shfl_xor_sync(0xffffffffu, acc1[t][2], 1), k0);
+            k1 = fmaf(frho, __shfl_xor_sync(0xffffffffu, acc1[t][3], 1), k1);
+            // (re, im) of one spin per lane: ri = 0 keeps its first column, ri = 1 its second
+            const float other = __shfl_xor_sync(0xffffffffu, ri ? k0 : k1, 4);
+            if (j < 3 && v < a.Nv) {
+                const cx<float> pc = unpack2(tc_lds<uint32_t>(ownw + 96 * t), (T*)nullptr);
+                const float dg = diag_of<float>(a, v);
+                const cx<float> o{fmaf(dg, pc.re, ri ? other : k0), fmaf(dg, pc.im, ri ? k1 : other)};
+                st_cs(op, pack2(o, (T*)nullptr));
             }
         }
     }
+    cp_async_wait<0>();
 }
 
-template <typename T, bool DAG>
-__global__ void __launch_bounds__(TC_THREADS, 1) k_brillouin_tc(ApplyArgs a, int nvb)
+template <typename T, int NT>
+cudaError_t tc_go_nt(bool dag, const ApplyArgs& a, int nvb, cudaStream_t st)
 {
-    extern __shared__ __align__(1024) unsigned char tc_smem[];
-    unsigned char* As = tc_smem + TC_A_OFF;
-    unsigned char* Bs = tc_smem + TC_B_OFF;
-    float* Ts = reinterpret_cast<float*>(tc_smem + TC_T_OFF);
-    const uint32_t bars = smem_u32(tc_smem + TC_BAR_OFF);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tc_smem + TC_BAR_OFF + 8 * TC_NBARS);
-    volatile int* abort = reinterpret_cast<volatile int*>(tc_smem + TC_BAR_OFF + 8 * TC_NBARS + 8);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-
-    // operands start at zero: K padding, vanishing classes, the d = 0 entries of B, absent rows
-    for (uint32_t i = tid; i < TC_T_OFF / 16; i += TC_THREADS)
-        reinterpret_cast<uint4*>(tc_smem)[i] = make_uint4(0u, 0u, 0u, 0u);
-    tc_fence_async();
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    }
-    if (tid == 0) {
-        for (int s = 0; s < TC_NS; ++s) {
-            tc_bar_init(bars + 8u * (TC_BAR_FA + s), TC_GTHREADS);   // the gatherers
-            tc_bar_init(bars + 8u * (TC_BAR_EA + s), 1);     // one commit
+    // the tile of at most 16 sites of a plane that fits two stages of shared memory and
+    // cuts the plane into the fewest tiles (16 x 16: 8 x 2), the smaller halo at equal counts
+    constexpr size_t room = 227 * 1024;
+    TcGrid G;
+    const int Lx = a.g.L[0], Ly = a.g.L[1];
+    long best = 0;
+    size_t smem = 0;
+    for (int bx = 1; bx <= TC_MAXW && bx <= Lx; ++bx)
+        for (int by = 1; bx * by <= TC_MAXW && by <= Ly; ++by) {
+            const size_t need = TC_TAB + (size_t)TC_STAGES * (bx * by * 27 * 48 + 3 * (bx + 2) * (by + 2) * (2 * NT * 48));
+            if (need > room) continue;
+            const long tiles = (long)((Lx + bx - 1) / bx) * ((Ly + by - 1) / by);
+            if (smem && (tiles > best || (tiles == best && need >= smem))) continue;
+            best = tiles;
+            smem = need;
+            G.bx = bx;
+            G.by = by;
         }
-        for (int b = 0; b < TC_NR; ++b) {
-            tc_bar_init(bars + 8u * (TC_BAR_FB + b), 3 * TC_BTHREADS);   // three sites' builders
-            tc_bar_init(bars + 8u * (TC_BAR_EB + b), 1);
-        }
-        for (int c = 0; c < TC_NACC; ++c) {
-            tc_bar_init(bars + 8u * (TC_BAR_FC + c), 1);
-            tc_bar_init(bars + 8u * (TC_BAR_EC + c), 128);   // the epilogue
-        }
-        tc_bar_init(bars + 8u * TC_BAR_DR, 1);
-        *abort = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *tmem_slot;
-    if (warp < TC_EPI_WARPS) {
-        // all accumulators start at zero (every MMA accumulates)
-        const uint32_t zero = 0u;
-        for (int c = 0; c < TC_NACC; ++c)
-            asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,"
-                         "%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};"
-                         ::"r"(tmem + 32u * c + ((uint32_t)(warp * 32) << 16)), "r"(zero) : "memory");
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-
-    if (warp < TC_EPI_WARPS) tc_epi_role<T>(a, nvb, smem_u32(Ts), tmem, bars, abort, tid);
-    else if (warp == TC_MMA_WARP) {
-        if (lane == 0) tc_mma_role<T>(a, nvb, smem_u32(As), smem_u32(Bs), tmem, bars, abort);
-    } else if (warp < TC_B_WARP0) {
-        tc_gather_role<T>(a, nvb, smem_u32(As), bars, abort, warp - TC_GATHER_WARP0, lane);
-    } else {
-        tc_b_role<T, DAG>(a, nvb, smem_u32(Bs), bars, abort, tid - TC_B_WARP0 * 32);
-    }
-
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (tid == 0 && *abort && a.err) atomicExch(a.err, (int)DIRAC_TIMEOUT);
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+    G.nvb = nvb;
+    G.nx = (Lx + G.bx - 1) / G.bx;
+    G.ny = (Ly + G.by - 1) / G.by;
+    G.fv = make_fdiv((uint32_t)nvb);
+    G.fx = make_fdiv((uint32_t)G.nx);
+    G.fy = make_fdiv((uint32_t)G.ny);
+    G.fw = make_fdiv((uint32_t)(G.bx + 2));
+    G.nitems = (a.nsites / a.g.stride[2]) * best * nvb;
+    if (G.nitems <= 0) return cudaSuccess;
+    if (G.nitems >= (1L << 31)) return cudaErrorInvalidValue;   // item numbers are 31 bits
+    const int threads = 32 * G.bx * G.by;
+    auto kern = k_brillouin_tc<T, NT>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    int dev = 0, nsm = 0, per = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads, smem)) != cudaSuccess) return e;
+    const long grid = std::min<long>(G.nitems, (long)nsm * std::max(per, 1));
+    const float rho = 64.f / 432.f;   // 4/27
+    kern<<<(unsigned)grid, threads, smem, st>>>(a, G, dag ? -rho : rho);
+    return cudaGetLastError();
 }
 
+// right-hand sides per item: Nv in equal blocks of at most 16, rounded up to 4, 8, 12 or 16
 template <typename T>
 cudaError_t tc_go(bool dag, const ApplyArgs& a, cudaStream_t st)
 {
-    static int nsm = 0;
-    if (!nsm) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0) nsm = 128;
+    const int nb = (a.Nv + 15) / 16, per = (a.Nv + nb - 1) / nb;
+    const int nt = (per + 3) / 4;
+    const int nvb = (a.Nv + 4 * nt - 1) / (4 * nt);
+    switch (nt) {
+    case 1: return tc_go_nt<T, 2>(dag, a, nvb, st);
+    case 2: return tc_go_nt<T, 4>(dag, a, nvb, st);
+    case 3: return tc_go_nt<T, 6>(dag, a, nvb, st);
+    default: return tc_go_nt<T, 8>(dag, a, nvb, st);
     }
-    auto kern = dag ? k_brillouin_tc<T, true> : k_brillouin_tc<T, false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
-    if (e != cudaSuccess) return e;
-    const int nvb = (a.Nv + TC_VB - 1) / TC_VB;
-    const long nitems = (a.nsites / a.g.L[0]) * (long)nvb;
-    // one CTA per SM: ~200 KB of shared memory and all 512 tensor-memory columns
-    const long grid = std::min<long>(nitems, nsm);
-    if (grid <= 0) return cudaSuccess;
-    kern<<<(unsigned)grid, TC_THREADS, TC_SMEM, st>>>(a, nvb);
-    return cudaGetLastError();
 }
 
 }  // namespace
@@ -760,60 +478,65 @@ cudaError_t brillouin_tc_prepare(cudaStream_t st)
     BriDir dirs[80];
     int reps[40];
     brillouin_tables(dirs, reps);
-    static const double rho[5] = {0.0, 64.0 / 432.0, 16.0 / 432.0, 4.0 / 432.0, 1.0 / 432.0};
-    TcDir t[80];
+    TcDir t[TC_SLOTS];
     int n = 0;
-    for (int g = 0; g < 3; ++g)
-        for (int r = 0; r < 27; ++r)
-            for (int j = 0; j < 80; ++j) {
-                const signed char* d = dirs[j].d;
-                if (d[0] + 1 != g || (d[1] + 1) + 3 * (d[2] + 1) + 9 * (d[3] + 1) != r) continue;
-                int k = 0;
-                for (int m = 0; m < 4; ++m) k += d[m] != 0;
-                TcDir& D = t[n++];
-                D.g = (signed char)g;
-                D.r = (signed char)r;
-                D.plane = (short)(dirs[j].neg ? 40 + dirs[j].rep : dirs[j].rep);
-                D.c0 = (float)dirs[j].a;   // -lambda_k / 2
-                D.rho = (float)rho[k];
-                D.nz = 0;
-                D.neg = 0;
-                for (int m = 0; m < 4; ++m) {
-                    D.nz |= (d[m] != 0) << m;
-                    D.neg |= (d[m] < 0) << m;
-                }
+    for (int ph = 0; ph < 3; ++ph)
+        for (int r = 0; r < 27; ++r) {
+            TcDir& D = t[n++];
+            const int d[4] = {r % 3 - 1, (r / 3) % 3 - 1, r / 9 - 1, tc_dt(ph)};
+            D.plane = -1;
+            D.k = 0;
+            for (int m = 0; m < 4; ++m) {
+                D.d[m] = (signed char)d[m];
+                D.k += d[m] != 0;
             }
-    if (n != 80) return cudaErrorInvalidValue;
+            for (int j = 0; j < 80; ++j)
+                if (dirs[j].d[0] == d[0] && dirs[j].d[1] == d[1] && dirs[j].d[2] == d[2] && dirs[j].d[3] == d[3])
+                    D.plane = (signed char)(dirs[j].neg ? 40 + dirs[j].rep : dirs[j].rep);
+        }
     e = cudaMemcpyToSymbolAsync(c_tc_dirs, t, sizeof(t), 0, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
     return e;
 }
 
-// the site-major copy: element (s, d, e) = W plane of direction d (tensor-core
-// order), entry e, at site s; 16-bit complex words copied unchanged
-__global__ void k_brillouin_tc_links(size_t vol, size_t nsite, const uint32_t* __restrict__ w80, uint32_t* __restrict__ wtc)
+// bytes of the site-major link copy
+size_t brillouin_tc_link_bytes(const Geom& g) { return (size_t)g.vol * TC_SLOTS * 48; }
+
+// The site-major copy: element (s, slot, c') = the words W[0][c'], W[1][c'],
+// W[2][c'], 0 of the direction of the slot (the centre: zeros).  A block takes 32
+// sites and a few slots through shared memory: reads along the sites, writes along
+// the elements of a site.
+constexpr int TCL_SLOTS = 9;
+__global__ void __launch_bounds__(256) k_brillouin_tc_links(size_t vol, const uint32_t* __restrict__ w80, uint4* __restrict__ wtc)
 {
-    const size_t n = nsite * 720;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t s = i / 720;
-        const int r = (int)(i - s * 720), d = r / 9, e = r - 9 * d;
-        wtc[i] = w80[blk_index(vol, 9, c_tc_dirs[d].plane, e, (long)s)];
+    __shared__ uint32_t sm[32][TCL_SLOTS * 9 + 1];
+    const long s0 = (long)blockIdx.x * 32;
+    const int sl0 = blockIdx.y * TCL_SLOTS;
+    for (int i = threadIdx.x; i < TCL_SLOTS * 9 * 32; i += 256) {
+        const int s = i & 31, se = i >> 5, sl = se / 9, e = se - 9 * sl;
+        const int plane = c_tc_dirs[sl0 + sl].plane;
+        sm[s][se] = (plane >= 0 && s0 + s < (long)vol) ? w80[blk_index(vol, 9, plane, e, s0 + s)] : 0u;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < TCL_SLOTS * 3 * 32; i += 256) {
+        const int s = i / (TCL_SLOTS * 3), r = i - s * (TCL_SLOTS * 3), sl = r / 3, q = r - 3 * sl;
+        if (s0 + s >= (long)vol) break;
+        const uint32_t* w = sm[s] + 9 * sl + q;
+        wtc[((size_t)(s0 + s) * TC_SLOTS + sl0 + sl) * 3 + q] = make_uint4(w[0], w[3], w[6], 0u);
     }
 }
 
 cudaError_t launch_brillouin_tc_links(const Geom& g, const void* w80, void* wtc, cudaStream_t st)
 {
-    const size_t nsite = nblk_of((size_t)g.vol) * 32;
-    const size_t n = nsite * 720;
-    const unsigned grid = (unsigned)std::min<size_t>((n + 255) / 256, 65535);
-    k_brillouin_tc_links<<<grid, 256, 0, st>>>((size_t)g.vol, nsite, static_cast<const uint32_t*>(w80),
-                                               static_cast<uint32_t*>(wtc));
+    static_assert(TC_SLOTS % TCL_SLOTS == 0, "whole groups of slots");
+    k_brillouin_tc_links<<<dim3((unsigned)nblk_of((size_t)g.vol), TC_SLOTS / TCL_SLOTS), 256, 0, st>>>(
+        (size_t)g.vol, static_cast<const uint32_t*>(w80), static_cast<uint4*>(wtc));
     return cudaGetLastError();
 }
 
-// a.links: the 80 W of each site, site-major in the order of c_tc_dirs
-// (launch_brillouin_tc_links), 16-bit; a.in, a.out 16-bit fields of the storage type
+// a.links: the W of each site, site-major (launch_brillouin_tc_links), 16-bit;
+// a.in, a.out 16-bit fields of the storage type
 cudaError_t launch_brillouin_tc(int prec, bool dag, const ApplyArgs& a, cudaStream_t st)
 {
     if (a.nsites == 0 || a.Nv == 0) return cudaSuccess;

@@ -393,7 +393,7 @@ dirac_status dirac_handle::build_link_alt()
         if ((st = cuda(launch_brillouin_w80(prec, g, links, links_alt, stream), "80-direction W"))) return st;
         if (prec != P_BF16 && prec != P_F16) return DIRAC_OK;
         // the copy the tensor-core sweep reads: the 80 W of a site in one piece
-        if (!links_tc && (st = alloc(&links_tc, nsite * 80 * 9 * cbytes(prec), "80-direction W, site-major"))) return st;
+        if (!links_tc && (st = alloc(&links_tc, brillouin_tc_link_bytes(g), "80-direction W, site-major"))) return st;
         return cuda(launch_brillouin_tc_links(g, links_alt, links_tc, stream), "80-direction W, site-major");
     }
     if (prec == P_F64)

@@ -38,7 +38,7 @@ enum Variant {
                     // site's own spinor (wilson_site_xlast, staggered_site_xlast); `block` =
                     // sites per block (32 or 64)
     V_TC = 7        // Brillouin, BF16/FP16 storage, link format 1: the per-site contraction on
-                    // the tensor cores (tcgen05.mma, apply_brillouin_tc.cu); R = 1, block = 128
+                    // the tensor cores (mma.sync, apply_brillouin_tc.cu); R = 1, block = 128
 };
 
 struct LaunchCfg {
@@ -97,6 +97,7 @@ cudaError_t brillouin_tc_prepare(cudaStream_t st);
 cudaError_t launch_brillouin_tc(int prec, bool dag, const ApplyArgs& a, cudaStream_t st);
 // the site-major copy of the 80 W (16-bit storage) the tensor-core sweep reads,
 // from link format 1 ([80][9][site], blocked); needs brillouin_tc_prepare
+size_t brillouin_tc_link_bytes(const Geom& g);
 cudaError_t launch_brillouin_tc_links(const Geom& g, const void* w80, void* wtc, cudaStream_t st);
 
 // Brillouin sweeps of the split inner solve (apply_brillouin_split.cuh):

@@ -355,6 +355,11 @@ static dirac_status apply_inner_whole(dirac_handle* h, SolverWS* w, bool dag, vo
     const void* L32 = nullptr;
     dirac_status st;
     if ((st = h->ensure_links32(&L32))) return st;
+    // a handle tuned to the tensor cores has no shape for these CUDA-core sweeps:
+    // three right-hand sides per thread, or two where the last group would be
+    // mostly empty (12^3 x 24, Nv = 12: 0.49 ms at R = 3, 0.67 ms at R = 1)
+    if (c0.variant == V_TC)
+        c0 = LaunchCfg{(w->W + 2) / 3 * 3 * 8 <= w->W * 9 ? 3 : 2, 128, V_DIRECT, std::min(8, h->g.L[3])};
     ApplyArgs a = h->args(out, in, w->W, h->diag);
     a.links = L32;
     a.diag_v = diag_v;
