@@ -191,6 +191,12 @@ DIRAC_API dirac_status dirac_apply_dagger(dirac_handle* h, void* out, const void
 DIRAC_API dirac_status dirac_force(dirac_handle* h, void* F, const void* psi, const void* g,
                                    dirac_layout layout);
 
+/* The whole backward pass of out = D psi for the cotangent g: gpsi = D^+ g
+ * (dirac_apply_dagger) and F (dirac_force), with g converted to the internal
+ * layout once.  All fields canonical, device; no two may be the same.
+ * Asynchronous. */
+DIRAC_API dirac_status dirac_backward(dirac_handle* h, void* gpsi, void* F, const void* psi, const void* g);
+
 /* Statistics of one dirac_solve call. */
 typedef struct {
     int outer_iterations;   /* refinement steps (inner solves) taken */

@@ -81,6 +81,7 @@ SIGNATURES = {
     "dirac_last_error": (ctypes.c_char_p, [P]),
     "dirac_solve": (I, [P, P, P, D, I, I, D, P, P]),
     "dirac_force": (I, [P, P, P, P, I]),
+    "dirac_backward": (I, [P, P, P, P, P]),
     "dirac_autotune": (I, [P, I, ctypes.POINTER(I), ctypes.POINTER(I), ctypes.POINTER(I), ctypes.POINTER(D)]),
     "dirac_solve_batched": (I, [P, I, P, P, P, P, D, I, I, D, P, P, P]),
     "dirac_apply_static": (I, [P, P, P, I]),
@@ -410,18 +411,34 @@ class Dirac:
 
     def force(self, psi, g, out=None):
         """Link gradient of Re <g, D psi>: canonical links shape, complex128 (f64) / complex64."""
-        torch = _torch()
-        Nx, Ny, Nz, Nt = self.L
         psi = self._canon_in(psi, "psi")
         g = self._canon_in(g, "g")
-        nl = Nx * Ny * Nz * Nt * 4 * self.Nc * self.Nc
-        if out is None:
-            out = torch.empty((Nt, Nz, Ny, Nx, 4, 3, 3), dtype=self.canon_dtype, device=self.device)
-        elif out.dtype != self.canon_dtype or not _is_device(out) or not out.is_contiguous() or out.numel() != nl:
-            raise ValueError(f"out must be a contiguous CUDA {self.canon_dtype} tensor with {nl} entries")
+        out = self._links_out(out)
         self._sync_stream()
         check(lib().dirac_force(self.h, _ptr(out), _ptr(psi), _ptr(g), CANONICAL), self.h, "dirac_force")
         return out
+
+    def _links_out(self, out=None):
+        torch = _torch()
+        Nx, Ny, Nz, Nt = self.L
+        nl = Nx * Ny * Nz * Nt * 4 * self.Nc * self.Nc
+        if out is None:
+            return torch.empty((Nt, Nz, Ny, Nx, 4, 3, 3), dtype=self.canon_dtype, device=self.device)
+        if out.dtype != self.canon_dtype or not _is_device(out) or not out.is_contiguous() or out.numel() != nl:
+            raise ValueError(f"out must be a contiguous CUDA {self.canon_dtype} tensor with {nl} entries")
+        return out
+
+    def backward(self, psi, g):
+        """(D^+ g, link gradient of Re <g, D psi>), as apply_dagger(g) and force(psi, g) give them."""
+        cls = type(self)
+        if cls.apply_dagger is not Dirac.apply_dagger or cls.force is not Dirac.force or cls.apply is not Dirac.apply:
+            return self.apply_dagger(g), self.force(psi, g)   # a subclass's own
+        psi = self._canon_in(psi, "psi")
+        g = self._canon_in(g, "g")
+        gpsi, F = self.new_canonical(), self._links_out()
+        self._sync_stream()
+        check(lib().dirac_backward(self.h, _ptr(gpsi), _ptr(F), _ptr(psi), _ptr(g)), self.h, "dirac_backward")
+        return gpsi, F
 
     def set_kernel_config(self, R: int, block: int, variant: int = 0):
         """Launch shape: R right-hand sides per thread, block, variant (0 direct,

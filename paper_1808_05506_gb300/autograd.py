@@ -47,9 +47,12 @@ class DiracApply(torch.autograd.Function):
         if D.links_generation != ctx.links_generation:
             D.set_links(V)   # the handle was given other links since the forward pass
         gpsi = gV = None
-        if ctx.needs_input_grad[0]:
+        if ctx.needs_input_grad[0] and ctx.needs_input_grad[1]:
+            gpsi, gV = D.backward(psi.detach(), g)
+            gpsi, gV = gpsi.to(psi.dtype), gV.to(V.dtype)
+        elif ctx.needs_input_grad[0]:
             gpsi = D.apply_dagger(g).to(psi.dtype)
-        if ctx.needs_input_grad[1]:
+        elif ctx.needs_input_grad[1]:
             gV = D.force(psi.detach().to(D.canon_dtype).contiguous(), g).to(V.dtype)
         return gpsi, gV, None, None
 

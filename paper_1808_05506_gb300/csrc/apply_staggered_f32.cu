@@ -1,0 +1,6 @@
+// Staggered sweep, FP32 storage (kernel templates in apply_staggered_impl.cuh).
+#include "apply_staggered_impl.cuh"
+
+namespace dirac {
+cudaError_t staggered_go_f32(bool dag, const ApplyArgs& a, LaunchCfg c, cudaStream_t st) { return staggered_go_T<float>(dag, a, c, st); }
+}  // namespace dirac

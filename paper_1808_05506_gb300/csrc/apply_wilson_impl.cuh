@@ -10,14 +10,22 @@
 namespace dirac {
 
 
-template <typename T, int R, bool DAG>
+// CANON: the output goes to the canonical field a.canon (warp_store, whole warps)
+template <typename T, int R, bool DAG, bool CANON>
 __global__ void __launch_bounds__(256) k_wilson(ApplyArgs a, int ngroups)
 {
     const long b = blockIdx.x;
     const int group = (int)(b % ngroups);
     const long p = (b / ngroups) * blockDim.x + threadIdx.x;
-    if (p >= a.nsites) return;
-    wilson_site<T, R, DAG>(a, slab_site(a, p), group);
+    if constexpr (CANON) {
+        extern __shared__ __align__(16) unsigned char sm[];
+        if (p - (threadIdx.x & 31) >= a.nsites) return;   // a whole warp
+        const OutTo to{sm + (threadIdx.x >> 5) * wilson_store_bytes<T>(), (int)(threadIdx.x & 31), p < a.nsites};
+        wilson_site<T, R, DAG, 0, 0, true>(a, slab_site(a, min(p, a.nsites - 1)), group, to);
+    } else {
+        if (p >= a.nsites) return;
+        wilson_site<T, R, DAG>(a, slab_site(a, p), group);
+    }
 }
 
 // V_TMARCH: blockDim = (sites, groups); a block owns a run of `block` site
@@ -70,20 +78,27 @@ __global__ void __launch_bounds__(256) k_wilson_pipe(ApplyArgs a, int ngroups)
 // V_GROUPS: blockDim = (sites, groups); block b covers a run of sites and a
 // chunk of gy right-hand-side groups
 // LF: link format (0 nine entries per link, 1 two rows, reconstructed)
-template <typename T, int R, bool DAG, int MODE, int LF>
+template <typename T, int R, bool DAG, int MODE, int LF, bool CANON>
 __global__ void __launch_bounds__(192, 2) k_wilson_groups(ApplyArgs a, int ngroups, int gy)
 {
     const int nchunks = (ngroups + gy - 1) / gy;
     const long b = blockIdx.x;
     const int group = (int)(b % nchunks) * gy + threadIdx.y;
     const long p = (b / nchunks) * blockDim.x + threadIdx.x;
-    if (p >= a.nsites || group >= ngroups) return;
-    wilson_site<T, R, DAG, MODE, LF>(a, slab_site(a, p), group);
+    if constexpr (CANON) {
+        __shared__ __align__(16) unsigned char sm[6][wilson_store_bytes<T>()];
+        if (p - (threadIdx.x & 31) >= a.nsites || group >= ngroups) return;   // a whole warp
+        const OutTo to{sm[(threadIdx.y * blockDim.x + threadIdx.x) >> 5], (int)(threadIdx.x & 31), p < a.nsites};
+        wilson_site<T, R, DAG, MODE, LF, true>(a, slab_site(a, min(p, a.nsites - 1)), group, to);
+    } else {
+        if (p >= a.nsites || group >= ngroups) return;
+        wilson_site<T, R, DAG, MODE, LF>(a, slab_site(a, p), group);
+    }
 }
 
 // V_XLAST: V_GROUPS with the x hops last, by lane exchange (wilson_site_xlast);
 // the host checked that every warp holds whole x-rows
-template <typename T, int R, bool DAG, int MODE, int LF>
+template <typename T, int R, bool DAG, int MODE, int LF, bool CANON>
 __global__ void __launch_bounds__(192, 2) k_wilson_xlast(ApplyArgs a, int ngroups, int gy)
 {
     const int nchunks = (ngroups + gy - 1) / gy;
@@ -91,7 +106,13 @@ __global__ void __launch_bounds__(192, 2) k_wilson_xlast(ApplyArgs a, int ngroup
     const int group = (int)(b % nchunks) * gy + threadIdx.y;
     const long p = (b / nchunks) * blockDim.x + threadIdx.x;
     if (p >= a.nsites || group >= ngroups) return;   // whole warps
-    wilson_site_xlast<T, R, DAG, MODE, LF>(a, slab_site(a, p), threadIdx.x & 31, group);
+    if constexpr (CANON) {
+        __shared__ __align__(16) unsigned char sm[6][wilson_store_bytes<T>()];
+        const OutTo to{sm[(threadIdx.y * blockDim.x + threadIdx.x) >> 5], (int)(threadIdx.x & 31), true};
+        wilson_site_xlast<T, R, DAG, MODE, LF, true>(a, slab_site(a, p), threadIdx.x & 31, group, to);
+    } else {
+        wilson_site_xlast<T, R, DAG, MODE, LF>(a, slab_site(a, p), threadIdx.x & 31, group);
+    }
 }
 
 template <typename T, int R>
@@ -99,6 +120,8 @@ cudaError_t go(bool dag, const ApplyArgs& a, LaunchCfg c, cudaStream_t st)
 {
     const int block = c.block;
     const int ngroups = (a.Nv + R - 1) / R;
+    // sweeps that write canonical fields (canon_supported)
+    constexpr bool CANON_BUILT = sizeof(T) >= 4 && R <= 2;
     const long nblk = ((a.nsites + block - 1) / block) * (long)ngroups;
     if constexpr (sizeof(T) != 8) {
     if (c.variant == V_GROUPS) {
@@ -110,8 +133,15 @@ cudaError_t go(bool dag, const ApplyArgs& a, LaunchCfg c, cudaStream_t st)
         auto launch_lf = [&](auto m, auto lf) {
             constexpr int M = decltype(m)::value;
             constexpr int LF = decltype(lf)::value;
-            if (dag) k_wilson_groups<T, R, true, M, LF><<<(unsigned)nb, dim3(block, gy), 0, st>>>(a, ngroups, gy);
-            else k_wilson_groups<T, R, false, M, LF><<<(unsigned)nb, dim3(block, gy), 0, st>>>(a, ngroups, gy);
+            if constexpr (CANON_BUILT && M < 2) {
+                if (a.canon) {
+                    if (dag) k_wilson_groups<T, R, true, M, LF, true><<<(unsigned)nb, dim3(block, gy), 0, st>>>(a, ngroups, gy);
+                    else k_wilson_groups<T, R, false, M, LF, true><<<(unsigned)nb, dim3(block, gy), 0, st>>>(a, ngroups, gy);
+                    return;
+                }
+            }
+            if (dag) k_wilson_groups<T, R, true, M, LF, false><<<(unsigned)nb, dim3(block, gy), 0, st>>>(a, ngroups, gy);
+            else k_wilson_groups<T, R, false, M, LF, false><<<(unsigned)nb, dim3(block, gy), 0, st>>>(a, ngroups, gy);
         };
         auto launch = [&](auto m) {
             if (c.fmt == 1) launch_lf(m, std::integral_constant<int, 1>{});
@@ -131,8 +161,15 @@ cudaError_t go(bool dag, const ApplyArgs& a, LaunchCfg c, cudaStream_t st)
         auto launch_lf = [&](auto m, auto lf) {
             constexpr int M = decltype(m)::value;
             constexpr int LF = decltype(lf)::value;
-            if (dag) k_wilson_xlast<T, R, true, M, LF><<<(unsigned)nb, dim3(block, gy), 0, st>>>(a, ngroups, gy);
-            else k_wilson_xlast<T, R, false, M, LF><<<(unsigned)nb, dim3(block, gy), 0, st>>>(a, ngroups, gy);
+            if constexpr (CANON_BUILT && M < 2) {
+                if (a.canon) {
+                    if (dag) k_wilson_xlast<T, R, true, M, LF, true><<<(unsigned)nb, dim3(block, gy), 0, st>>>(a, ngroups, gy);
+                    else k_wilson_xlast<T, R, false, M, LF, true><<<(unsigned)nb, dim3(block, gy), 0, st>>>(a, ngroups, gy);
+                    return;
+                }
+            }
+            if (dag) k_wilson_xlast<T, R, true, M, LF, false><<<(unsigned)nb, dim3(block, gy), 0, st>>>(a, ngroups, gy);
+            else k_wilson_xlast<T, R, false, M, LF, false><<<(unsigned)nb, dim3(block, gy), 0, st>>>(a, ngroups, gy);
         };
         auto launch = [&](auto m) {
             if (c.fmt == 1) launch_lf(m, std::integral_constant<int, 1>{});
@@ -172,8 +209,16 @@ cudaError_t go(bool dag, const ApplyArgs& a, LaunchCfg c, cudaStream_t st)
         return cudaGetLastError();
     }
     }   // not FP64
-    if (dag) k_wilson<T, R, true><<<(unsigned)nblk, block, 0, st>>>(a, ngroups);
-    else k_wilson<T, R, false><<<(unsigned)nblk, block, 0, st>>>(a, ngroups);
+    if constexpr (CANON_BUILT) {
+        if (a.canon) {
+            const size_t sm = (size_t)(block / 32) * wilson_store_bytes<T>();
+            if (dag) k_wilson<T, R, true, true><<<(unsigned)nblk, block, sm, st>>>(a, ngroups);
+            else k_wilson<T, R, false, true><<<(unsigned)nblk, block, sm, st>>>(a, ngroups);
+            return cudaGetLastError();
+        }
+    }
+    if (dag) k_wilson<T, R, true, false><<<(unsigned)nblk, block, 0, st>>>(a, ngroups);
+    else k_wilson<T, R, false, false><<<(unsigned)nblk, block, 0, st>>>(a, ngroups);
     return cudaGetLastError();
 }
 

@@ -127,7 +127,7 @@ ApplyArgs dirac_handle::args(void* out, const void* in, int nv, double diag_valu
 
 dirac_status dirac_handle::run_apply(bool dagger, void* out, const void* in, int nv,
                                      double diag_value, const void* link_ptr, int p, LaunchCfg c,
-                                     const double* diag_v, int t0, int nt, const float* diag_vf)
+                                     const double* diag_v, int t0, int nt, const float* diag_vf, void* canon)
 {
     // link format 1 (dirac_set_link_format) for the storage links, where the
     // launch variant reads it; every other call reads the plain links
@@ -145,6 +145,7 @@ dirac_status dirac_handle::run_apply(bool dagger, void* out, const void* in, int
     a.links = link_ptr;
     a.diag_v = diag_v;
     a.diag_vf = diag_vf;
+    a.canon = canon;
     a.err = dev_err;
     if (nt > 0) {   // the slab of nt t-slices from t0 (variants 0, 1, 2 and 5)
         a.t0 = t0;
@@ -157,6 +158,16 @@ dirac_status dirac_handle::run_apply(bool dagger, void* out, const void* in, int
         a.fdt = make_fdiv((uint32_t)a.tc);
     }
     return cuda(launch_apply(op, p, dagger, a, c, stream), "apply kernel launch");
+}
+
+// the canonical result of a packed field: written by the sweep where it can, else
+// through ws_out
+dirac_status dirac_handle::run_apply_canonical(bool dagger, void* out, const void* in)
+{
+    const bool direct = canon_supported(op, prec, cfg);
+    const dirac_status st = run_apply(dagger, ws_out, in, Nv, diag, links, prec, cfg, nullptr, 0, 0, nullptr,
+                                      direct ? out : nullptr);
+    return st || direct ? st : dirac_unpack(this, out, ws_out);
 }
 
 static bool is_device_ptr(const void* p)
@@ -327,15 +338,19 @@ dirac_status dirac_set_links(dirac_handle* h, const void* V, dirac_prec V_prec, 
         h->release(dV);
         return st;
     }
-    st = h->cuda(launch_links_to_f64(h->g, src, f64, h->links64, h->stream), "links conversion");
+    const int nmat = (h->op == OP_BRILLOUIN) ? 40 : 4;
+    if (!h->links &&
+        (st = h->alloc(&h->links, nblk_of((size_t)h->g.vol) * 32 * 9 * nmat * cbytes(h->prec), "links"))) {
+        h->release(dV);
+        return st;
+    }
+    st = h->cuda(launch_links_load(h->g, src, f64, h->links64, h->op == OP_BRILLOUIN ? -1 : h->prec, h->links, h->stream),
+                 "links conversion");
     h->release_after_sync(dV);
     if (st) return st;
     h->release(h->W64);
     h->release(h->links64b);
     h->release(h->links_df);
-    const int nmat = (h->op == OP_BRILLOUIN) ? 40 : 4;
-    if (!h->links && (st = h->alloc(&h->links, nblk_of((size_t)h->g.vol) * 32 * 9 * nmat * cbytes(h->prec), "links")))
-        return st;
     if (h->op == OP_BRILLOUIN) {
         if (h->prec == P_F64) {
             if ((st = h->build_W64())) return st;
@@ -356,8 +371,6 @@ dirac_status dirac_set_links(dirac_handle* h, const void* V, dirac_prec V_prec, 
         }
         if (st) return st;
     } else {
-        st = h->cuda(launch_convert_links(h->prec, h->g, 4, h->links64, h->links, h->stream), "links conversion");
-        if (st) return st;
         // the FP32 copy of the split inner solve is refreshed in place, like the
         // storage links: a captured solver graph holds both addresses
         if (h->links32 && h->links32 != h->links) {
@@ -588,9 +601,7 @@ static dirac_status apply_common(dirac_handle* h, bool dagger, void* out, const 
         return h->run_apply(dagger, out, in, h->Nv, h->diag, h->links, h->prec, h->cfg);
     if ((st = h->ensure_workspace())) return st;
     if ((st = dirac_pack(h, h->ws_in, in))) return st;
-    if ((st = h->run_apply(dagger, h->ws_out, h->ws_in, h->Nv, h->diag, h->links, h->prec, h->cfg)))
-        return st;
-    return dirac_unpack(h, out, h->ws_out);
+    return h->run_apply_canonical(dagger, out, h->ws_in);
 }
 
 dirac_status dirac_apply(dirac_handle* h, void* out, const void* in, dirac_layout layout)

@@ -320,6 +320,47 @@ DEV_INLINE void store_spinor(void* base, size_t vol, int v, long s, const cx<typ
     }
 }
 
+// a value as the storage type T holds it (16-bit types round)
+template <typename T> DEV_INLINE cx<typename Store<T>::A> stored_value(cx<typename Store<T>::A> c)
+{
+    if constexpr (sizeof(T) == 2) return unpack2(pack2(c, (T*)nullptr), (T*)nullptr);
+    else return c;
+}
+
+// Canonical output of a sweep (FP32 and FP64 storage): the N units (16 bytes, or
+// the 8-byte complex of an FP32 staggered spinor) that each lane of a warp holds for
+// its site go to dst[s * row + off .. + N - 1].  Through N + 1 units of shared memory per
+// lane, so that the warp writes runs of N units; a lane writing its own site's would touch
+// 32 runs with every store (16^4, Nv = 8, FP32 Wilson: the sweep took 52 us that way,
+// 41 us with internal output, and the separate pass to canonical fields it saves 20 us).
+// Every lane of the warp calls this; valid: the lane has a site.
+template <int N, typename U>
+DEV_INLINE void warp_store(U* sm, U* dst, size_t row, size_t off, int s, bool valid, int lane, const U* val)
+{
+#if defined(__CUDA_ARCH__)
+    constexpr int PITCH = N | 1;
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < N; ++u) sm[lane * PITCH + u] = val[u];
+    __syncwarp();
+    const int sv = valid ? s : -1;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const int c = i * 32 + lane, j = c / N, u = c - j * N;
+        const int sj = __shfl_sync(0xffffffffu, sv, j);
+        if (sj >= 0) __stcs(dst + (size_t)sj * row + off + u, sm[j * PITCH + u]);
+    }
+#else
+    (void)sm; (void)dst; (void)row; (void)off; (void)s; (void)valid; (void)lane; (void)val;
+#endif
+}
+DEV_INLINE float4 unit2(cx<float> a, cx<float> b) { return make_float4(a.re, a.im, b.re, b.im); }
+DEV_INLINE float2 unit1(cx<float> a) { return make_float2(a.re, a.im); }
+DEV_INLINE double2 unit1(cx<double> a) { return make_double2(a.re, a.im); }
+// units of shared memory per warp for R staggered right-hand sides, and bytes for Wilson
+template <typename T> constexpr int wilson_store_bytes() { return 32 * (sizeof(T) == 8 ? 13 : 7) * 16; }
+template <typename T, int R> constexpr int staggered_store_bytes() { return 32 * ((3 * R) | 1) * 2 * (int)sizeof(T); }
+
 // the same loads with an L1 policy (NA: do not allocate in L1)
 template <typename T, bool NA> DEV_INLINE cx<typename Store<T>::A> ld_one_p(const void* base, size_t i)
 {
@@ -473,6 +514,25 @@ DEV_INLINE void mat_dag_vec_acc2(const cx<float>* U, const cx<float>* h, cx<floa
             acc[a] = {r.x, r.y};
         }
     }
+}
+
+// v with its sign flipped where bit 31 of m is set (no arithmetic: the FP64 pipe
+// of this GPU is 62 times slower than the integer one)
+HD float flip_sign(float v, uint32_t m)
+{
+#if defined(__CUDA_ARCH__)
+    return __uint_as_float(__float_as_uint(v) ^ m);
+#else
+    return (m & 0x80000000u) ? -v : v;
+#endif
+}
+HD double flip_sign(double v, uint32_t m)
+{
+#if defined(__CUDA_ARCH__)
+    return __hiloint2double(__double2hiint(v) ^ (int)m, __double2loint(v));
+#else
+    return (m & 0x80000000u) ? -v : v;
+#endif
 }
 
 // value of v held by lane src of this warp (all 32 lanes take part)

@@ -50,13 +50,6 @@ struct EoArgs {
 // partials per column of the fused norm of a sweep with `block` half sites per block
 inline long eo_norm_slots(long vh, int block) { return ((vh + block - 1) / block) * (block / 32); }
 
-// a value as the storage type T holds it (16-bit types round)
-template <typename T> DEV_INLINE cx<typename Store<T>::A> stored_value(cx<typename Store<T>::A> c)
-{
-    if constexpr (sizeof(T) == 2) return unpack2(pack2(c, (T*)nullptr), (T*)nullptr);
-    else return c;
-}
-
 // site of parity a.par with half-site index h
 HD long eo_site(const EoArgs& a, long h)
 {
@@ -167,7 +160,7 @@ DEV_INLINE void staggered_eo_site(const EoArgs& a, long h, int group, typename S
     int par = 0;  // x_0 + ... + x_{mu-1}
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
-        const A eta = (par & 1) ? A(-1) : A(1);
+        const uint32_t eta = (uint32_t)par << 31;
         par += x[mu];
         cx<A> Uf[9], Ub[9];
         load_link<TL>(a.links, a.g.vol, mu, s, Uf);
@@ -175,17 +168,10 @@ DEV_INLINE void staggered_eo_site(const EoArgs& a, long h, int group, typename S
         const long hf = (s + fwd[mu]) >> 1, hb = (s + bwd[mu]) >> 1;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            cx<A> pf[3], pb[3], w[3] = {}, wb[3] = {};
+            cx<A> pf[3], pb[3];
             load_spinor<TI, 3>(a.in, a.vh, v0 + r, hf, pf);
             load_spinor<TI, 3>(a.in, a.vh, v0 + r, hb, pb);
-            mat_vec(Uf, pf, w);
-            mat_dag_vec(Ub, pb, wb);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                cx<A> d = w[c] - wb[c];
-                acc[r][c].re = fma(eta, d.re, acc[r][c].re);
-                acc[r][c].im = fma(eta, d.im, acc[r][c].im);
-            }
+            staggered_hops(Uf, Ub, pf, pb, mu == 0 ? 0u : eta, acc[r]);
         }
     }
     const A* cf = static_cast<const A*>(a.coef);

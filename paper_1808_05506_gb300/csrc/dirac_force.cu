@@ -11,7 +11,7 @@
 //     h = a_up + S B a_down, k = b_up + S B b_down.
 //   staggered (Sec. 3; eta_mu(x + mu) = eta_mu(x)):
 //     F_mu(x) = 1/2 eta_mu(x) sum_v [g_v(x) psi_v(x+mu)^+ - psi_v(x) g_v(x+mu)^+]
-// One thread owns one link (x, mu), gathers both hops that touch it and
+// One thread owns NM links of one site, gathers both hops that touch each and
 // writes it once (no atomics).  The Brillouin gradient, through the composite
 // transporters W, is in dirac_force_brillouin.cu.
 #include "dirac_handle.h"
@@ -21,95 +21,171 @@ using namespace dirac;
 
 namespace dirac {
 
-// acc[a][b] += c * sum_{comp} u_comp[a] conj(w_comp[b]) for ncomp 3-vectors
-template <typename A>
-__device__ __forceinline__ void outer_acc(cx<A>* acc, const cx<A>* u, const cx<A>* w, int ncomp, A c)
+// acc[a][b] += sum_{comp} u_comp[a] conj(w_comp[b]) for NC 3-vectors
+template <int NC, typename A>
+__device__ __forceinline__ void outer_acc(cx<A>* acc, const cx<A>* u, const cx<A>* w)
 {
-    for (int k = 0; k < ncomp; ++k)
+#pragma unroll
+    for (int k = 0; k < NC; ++k)
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
-            for (int b = 0; b < 3; ++b) {
-                cx<A> t = cfma_conj(w[3 * k + b], u[3 * k + a], cx<A>{A(0), A(0)});   // u conj(w)
-                acc[3 * a + b].re = fma(c, t.re, acc[3 * a + b].re);
-                acc[3 * a + b].im = fma(c, t.im, acc[3 * a + b].im);
-            }
+            for (int b = 0; b < 3; ++b) acc[3 * a + b] = cfma_conj(w[3 * k + b], u[3 * k + a], acc[3 * a + b]);
 }
 
-template <typename T, int MU>
-__device__ __forceinline__ void wilson_force_link(const Geom& g, int Nv, const void* psi, const void* gv,
-                                                  long s, long sp, cx<typename Store<T>::A>* acc)
+// acc += t (FP32), the products having gone into t; FP64: t is acc
+template <int NC, typename A>
+__device__ __forceinline__ void outer_sum(cx<A>* acc, const cx<A>* u, const cx<A>* w, const cx<A>* u2, const cx<A>* w2)
+{
+    if constexpr (sizeof(A) == 8) {
+        outer_acc<NC>(acc, u, w);
+        outer_acc<NC>(acc, u2, w2);
+    } else {
+        cx<A> t[9];
+#pragma unroll
+        for (int e = 0; e < 9; ++e) t[e] = cx<A>{A(0), A(0)};
+        outer_acc<NC>(t, u, w);
+        outer_acc<NC>(t, u2, w2);
+#pragma unroll
+        for (int e = 0; e < 9; ++e) acc[e] = acc[e] + t[e];
+    }
+}
+
+template <int MU, typename A>
+__device__ __forceinline__ void wilson_force_hop(cx<A>* acc, const cx<A>* gs, const cx<A>* ps, const cx<A>* gn, const cx<A>* pn)
+{
+    cx<A> h[6], k[6], h2[6], k2[6];
+    wilson_project<MU, -1>(gs, h);
+    wilson_project<MU, -1>(pn, k);
+    wilson_project<MU, +1>(ps, k2);
+    wilson_project<MU, +1>(gn, h2);
+    outer_sum<2>(acc, h, k, k2, h2);
+}
+
+// The links mu = m0 .. m0 + NM - 1 of site s.  The four links of a site share
+// psi(x) and g(x): NM links in a thread load 2 + 2 NM spinors per right-hand
+// side instead of 4 NM.  FP32 and 16-bit: bound by those loads, which come from
+// L2 (16 a site at NM = 1; 16^4, Nv = 8, FP32 Wilson: NM = 1 61 us, 2 55, 4 43).  Each hop's products are
+// summed by themselves before they join the sum over right-hand sides (a chain
+// of all of them in FP32 rounds more).  FP64: bound by FP64 arithmetic,
+// 72 multiply-adds per link, right-hand side and colour pair of spinors, so the
+// products go straight into the sums and the factor -1/2 (eta / 2) to the end
+// (staggered 404 -> 265 us).
+template <typename T, int M0, int NM>
+__device__ __forceinline__ void wilson_force_links(const Geom& g, int Nv, const void* psi, const void* gv, long s,
+                                                   const long* fwd, cx<typename Store<T>::A> (&acc)[NM][9])
 {
     using A = typename Store<T>::A;
     for (int v = 0; v < Nv; ++v) {
-        cx<A> a[12], b[12], h[6], k[6];
-        load_spinor<T, 12>(gv, g.vol, v, s, a);
-        load_spinor<T, 12>(psi, g.vol, v, sp, b);
-        wilson_project<MU, -1>(a, h);
-        wilson_project<MU, -1>(b, k);
-        outer_acc(acc, h, k, 2, A(-0.5));
-        load_spinor<T, 12>(psi, g.vol, v, s, a);
-        load_spinor<T, 12>(gv, g.vol, v, sp, b);
-        wilson_project<MU, +1>(a, k);
-        wilson_project<MU, +1>(b, h);
-        outer_acc(acc, k, h, 2, A(-0.5));
+        cx<A> gs[12], ps[12], gn[12], pn[12];
+        load_spinor<T, 12>(gv, g.vol, v, s, gs);
+        load_spinor<T, 12>(psi, g.vol, v, s, ps);
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {
+            load_spinor<T, 12>(gv, g.vol, v, s + fwd[M0 + m], gn);
+            load_spinor<T, 12>(psi, g.vol, v, s + fwd[M0 + m], pn);
+            if (M0 + m == 0) wilson_force_hop<0>(acc[m], gs, ps, gn, pn);
+            else if (M0 + m == 1) wilson_force_hop<1>(acc[m], gs, ps, gn, pn);
+            else if (M0 + m == 2) wilson_force_hop<2>(acc[m], gs, ps, gn, pn);
+            else wilson_force_hop<3>(acc[m], gs, ps, gn, pn);
+        }
     }
 }
 
-template <typename T, bool STAG>
+template <typename T, bool STAG, int NM>
 __global__ void __launch_bounds__(128) k_force(Geom g, int Nv, const void* psi, const void* gv, void* F)
 {
     using A = typename Store<T>::A;
-    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;   // (mu, site), site fastest
-    if (i >= 4 * g.vol) return;
-    const long s = i % g.vol;
-    const int mu = (int)(i / g.vol);
+    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;   // (links of a site, site), site fastest
+    if (i >= (4 / NM) * g.vol) return;
+    const int q = (int)(i / g.vol), m0 = q * NM;
+    const long s = i - q * g.vol;
     long fwd[4], bwd[4];
     int x[4];
     site_offsets(g, s, fwd, bwd, x);
-    const long sp = s + fwd[mu];
-    cx<A> acc[9];
+    cx<A> acc[NM][9];
 #pragma unroll
-    for (int e = 0; e < 9; ++e) acc[e] = cx<A>{A(0), A(0)};
+    for (int m = 0; m < NM; ++m)
+#pragma unroll
+        for (int e = 0; e < 9; ++e) acc[m][e] = cx<A>{A(0), A(0)};
+    A f[NM];
     if constexpr (STAG) {
-        int par = 0;
-        for (int nu = 0; nu < mu; ++nu) par += x[nu];
-        const A eta = (par & 1) ? A(-0.5) : A(0.5);
+        long sp[NM];
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {
+            const int mu = m0 + m;
+            const int par = (mu > 0 ? x[0] : 0) + (mu > 1 ? x[1] : 0) + (mu > 2 ? x[2] : 0);
+            f[m] = (par & 1) ? A(-0.5) : A(0.5);
+            sp[m] = s + (mu == 0 ? fwd[0] : (mu == 1 ? fwd[1] : (mu == 2 ? fwd[2] : fwd[3])));
+        }
         for (int v = 0; v < Nv; ++v) {
-            cx<A> a[3], b[3];
-            load_spinor<T, 3>(gv, g.vol, v, s, a);
-            load_spinor<T, 3>(psi, g.vol, v, sp, b);
-            outer_acc(acc, a, b, 1, eta);
-            load_spinor<T, 3>(psi, g.vol, v, s, a);
-            load_spinor<T, 3>(gv, g.vol, v, sp, b);
-            outer_acc(acc, a, b, 1, -eta);
+            cx<A> gs[3], ps[3], gn[3], pn[3];
+            load_spinor<T, 3>(gv, g.vol, v, s, gs);
+            load_spinor<T, 3>(psi, g.vol, v, s, ps);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) ps[c] = -ps[c];
+#pragma unroll
+            for (int m = 0; m < NM; ++m) {
+                load_spinor<T, 3>(gv, g.vol, v, sp[m], gn);
+                load_spinor<T, 3>(psi, g.vol, v, sp[m], pn);
+                outer_sum<1>(acc[m], gs, pn, ps, gn);
+            }
         }
     } else {
-        switch (mu) {
-        case 0: wilson_force_link<T, 0>(g, Nv, psi, gv, s, sp, acc); break;
-        case 1: wilson_force_link<T, 1>(g, Nv, psi, gv, s, sp, acc); break;
-        case 2: wilson_force_link<T, 2>(g, Nv, psi, gv, s, sp, acc); break;
-        default: wilson_force_link<T, 3>(g, Nv, psi, gv, s, sp, acc); break;
+#pragma unroll
+        for (int m = 0; m < NM; ++m) f[m] = A(-0.5);
+        if constexpr (NM == 4) wilson_force_links<T, 0, 4>(g, Nv, psi, gv, s, fwd, acc);
+        else if constexpr (NM == 2) {
+            if (q == 0) wilson_force_links<T, 0, 2>(g, Nv, psi, gv, s, fwd, acc);
+            else wilson_force_links<T, 2, 2>(g, Nv, psi, gv, s, fwd, acc);
+        } else {
+            if (q == 0) wilson_force_links<T, 0, 1>(g, Nv, psi, gv, s, fwd, acc);
+            else if (q == 1) wilson_force_links<T, 1, 1>(g, Nv, psi, gv, s, fwd, acc);
+            else if (q == 2) wilson_force_links<T, 2, 1>(g, Nv, psi, gv, s, fwd, acc);
+            else wilson_force_links<T, 3, 1>(g, Nv, psi, gv, s, fwd, acc);
         }
     }
-    using O = typename Store<A>::One;   // float2 or double2
-    O* out = reinterpret_cast<O*>(F) + ((size_t)s * 4 + mu) * 9;
+    if constexpr (sizeof(A) == 4 && NM > 1) {
+        // the NM links of a site are 72 NM contiguous bytes, 16-byte aligned for even NM
+        float4* out = reinterpret_cast<float4*>(static_cast<float2*>(F) + ((size_t)s * 4 + m0) * 9);
 #pragma unroll
-    for (int e = 0; e < 9; ++e) {
-        O o;
-        o.x = acc[e].re;
-        o.y = acc[e].im;
-        out[e] = o;
+        for (int e = 0; e < NM * 9; e += 2) {
+            const cx<A> c0 = acc[e / 9][e % 9], c1 = acc[(e + 1) / 9][(e + 1) % 9];
+            const A f0 = f[e / 9], f1 = f[(e + 1) / 9];
+            out[e / 2] = make_float4(f0 * c0.re, f0 * c0.im, f1 * c1.re, f1 * c1.im);
+        }
+    } else {
+        using O = typename Store<A>::One;   // float2 or double2
+        O* out = reinterpret_cast<O*>(F) + ((size_t)s * 4 + m0) * 9;
+#pragma unroll
+        for (int e = 0; e < NM * 9; ++e) {
+            O o;
+            o.x = f[e / 9] * acc[e / 9][e % 9].re;
+            o.y = f[e / 9] * acc[e / 9][e % 9].im;
+            out[e] = o;
+        }
     }
 }
 
+template <typename T, bool STAG, int NM>
+static cudaError_t force_go(const Geom& g, int Nv, const void* psi, const void* gv, void* F, cudaStream_t st)
+{
+    const long n = (4 / NM) * g.vol;
+    k_force<T, STAG, NM><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(g, Nv, psi, gv, F);
+    return cudaGetLastError();
+}
+
+// links per thread: FP64 one (144 registers of sums for four)
 template <typename T>
 static cudaError_t force_T(int op, const Geom& g, int Nv, const void* psi, const void* gv, void* F, cudaStream_t st)
 {
-    const unsigned nb = (unsigned)((4 * g.vol + 127) / 128);
-    if (op == OP_STAGGERED) k_force<T, true><<<nb, 128, 0, st>>>(g, Nv, psi, gv, F);
-    else k_force<T, false><<<nb, 128, 0, st>>>(g, Nv, psi, gv, F);
-    return cudaGetLastError();
+    if constexpr (sizeof(T) == 8) {
+        if (op == OP_STAGGERED) return force_go<T, true, 1>(g, Nv, psi, gv, F, st);
+        return force_go<T, false, 1>(g, Nv, psi, gv, F, st);
+    } else {
+        if (op == OP_STAGGERED) return force_go<T, true, 4>(g, Nv, psi, gv, F, st);
+        return force_go<T, false, 4>(g, Nv, psi, gv, F, st);
+    }
 }
 
 cudaError_t launch_force(int op, int prec, const Geom& g, int Nv, const void* psi, const void* gv, void* F,
@@ -125,6 +201,24 @@ cudaError_t launch_force(int op, int prec, const Geom& g, int Nv, const void* ps
 }
 
 }  // namespace dirac
+
+// the link gradient from packed fields
+static dirac_status force_internal(dirac_handle* h, void* F, const void* pi, const void* gi)
+{
+    if (h->op != OP_BRILLOUIN)
+        return h->cuda(launch_force(h->op, h->prec, h->g, h->Nv, pi, gi, F, h->stream), "force kernel launch");
+    // the transporters are rebuilt from V (not kept from the forward pass): 40
+    // planes of W and 81 of G
+    const size_t plane = (size_t)h->g.vol * 9 * 16;
+    void* scr = nullptr;
+    dirac_status st;
+    if ((st = h->scratch(121 * plane, &scr))) return st;
+    st = h->cuda(launch_force_brillouin(h->prec, h->g, h->Nv, pi, gi, h->links64, scr,
+                                        static_cast<char*>(scr) + 40 * plane, F, h->stream),
+                 "Brillouin force kernels");
+    h->scratch_done();
+    return st;
+}
 
 extern "C" DIRAC_API dirac_status dirac_force(dirac_handle* h, void* F, const void* psi, const void* g,
                                               dirac_layout layout)
@@ -145,17 +239,22 @@ extern "C" DIRAC_API dirac_status dirac_force(dirac_handle* h, void* F, const vo
         pi = h->ws_in;
         gi = h->ws_out;
     }
-    if (h->op == OP_BRILLOUIN) {
-        // the transporters are rebuilt from V (not kept from the forward pass):
-        // 40 planes of W and 81 of G
-        const size_t plane = (size_t)h->g.vol * 9 * 16;
-        void* scr = nullptr;
-        if ((st = h->scratch(121 * plane, &scr))) return st;
-        st = h->cuda(launch_force_brillouin(h->prec, h->g, h->Nv, pi, gi, h->links64, scr,
-                                            static_cast<char*>(scr) + 40 * plane, F, h->stream),
-                     "Brillouin force kernels");
-        h->scratch_done();
-        return st;
-    }
-    return h->cuda(launch_force(h->op, h->prec, h->g, h->Nv, pi, gi, F, h->stream), "force kernel launch");
+    return force_internal(h, F, pi, gi);
+}
+
+extern "C" DIRAC_API dirac_status dirac_backward(dirac_handle* h, void* gpsi, void* F, const void* psi, const void* g)
+{
+    if (!h) return DIRAC_ERR_INVALID_ARG;
+    if (!gpsi || !F || !psi || !g || gpsi == psi || gpsi == g || F == psi || F == g || F == gpsi)
+        return h->fail(DIRAC_ERR_INVALID_ARG, "dirac_backward: NULL or aliased pointers");
+    if (!h->have_links) return h->fail(DIRAC_ERR_INVALID_ARG, "dirac_backward: call dirac_set_links first");
+    if (!dirac_check_device_ptr(gpsi) || !dirac_check_device_ptr(F) || !dirac_check_device_ptr(psi) ||
+        !dirac_check_device_ptr(g))
+        return h->fail(DIRAC_ERR_INVALID_ARG, "dirac_backward: need 16-byte aligned device pointers");
+    dirac_status st;
+    if ((st = h->ensure_workspace())) return st;
+    if ((st = dirac_pack(h, h->ws_in, g))) return st;
+    if ((st = h->run_apply_canonical(true, gpsi, h->ws_in))) return st;   // may pass through ws_out
+    if ((st = dirac_pack(h, h->ws_out, psi))) return st;
+    return force_internal(h, F, h->ws_out, h->ws_in);
 }

@@ -60,6 +60,18 @@ inline bool link_format_supported(int op, int prec, int variant)
     return prec != P_F64 && (variant == V_GROUPS || variant == V_XLAST);
 }
 
+// whether the sweep of this launch shape can write a canonical field itself
+// (ApplyArgs::canon): FP32 and FP64, whose canonical numbers are the stored ones
+inline bool canon_supported(int op, int prec, const LaunchCfg& c)
+{
+    if (prec != P_F32 && prec != P_F64) return false;
+    if (op == OP_BRILLOUIN) return false;   // its pack and unpack are 4 % of a sweep
+    if (c.variant != V_DIRECT && c.variant != V_GROUPS && c.variant != V_XLAST) return false;
+    // FP64 blocks whose warps would gather their runs in more than 48 KB of shared memory
+    if (prec == P_F64 && c.variant == V_DIRECT && c.block > 128) return false;
+    return op == OP_WILSON ? c.R <= 2 : (prec == P_F32 || c.R < 6);
+}
+
 // threads per block of V_GROUPS: block sites x gy groups with block * gy <= 192
 inline int groups_per_block(int block, int ngroups)
 {
@@ -126,9 +138,10 @@ cudaError_t launch_pack_column64(int nsc, const Geom& g, int Nsrc, int c, const 
 cudaError_t launch_unpack_column64(int nsc, const Geom& g, int v, const void* internal, int Nsrc, int c, void* canon,
                                    cudaStream_t st);
 
-// canonical links V[s][mu][a][b] -> FP64 internal [mu][9][s]
-cudaError_t launch_links_to_f64(const Geom& g, const void* canon, bool canon_f64, void* V64,
-                                cudaStream_t st);
+// canonical links V[s][mu][a][b] -> FP64 internal [mu][9][s] and, for prec >= 0, the
+// storage links dst in that precision
+cudaError_t launch_links_load(const Geom& g, const void* canon, bool canon_f64, void* V64, int prec, void* dst,
+                              cudaStream_t st);
 // FP64 internal [m][9][s] -> storage precision internal [m][9][s] (nmat matrices per site)
 cudaError_t launch_convert_links(int prec, const Geom& g, int nmat, const void* src64, void* dst,
                                  cudaStream_t st);

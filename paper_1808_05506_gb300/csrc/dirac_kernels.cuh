@@ -34,6 +34,7 @@ struct ApplyArgs {
     int Nv;
     const void* in;       // internal spinor layout
     void* out;            // internal spinor layout
+    void* canon = nullptr;   // the output of the sweeps that write a canonical field (whole lattice)
     const void* links;    // internal link layout (V_mu or the 40 stored W)
     double diag;          // (4 + m0) Wilson, m staggered, (m0 + 15/8) Brillouin
     const double* diag_v; // per-right-hand-side diagonal (device, Nv entries) or null: diag for all
@@ -58,6 +59,56 @@ template <typename A> DEV_INLINE A diag_of(const ApplyArgs& a, int v)
 {
     if constexpr (sizeof(A) == 4) return a.diag_vf ? a.diag_vf[v] : (a.diag_v ? (A)a.diag_v[v] : a.diagf);
     else return a.diag_v ? a.diag_v[v] : a.diag;
+}
+
+// Where a sweep's result goes: the internal field a.out, or (CANON) the canonical
+// field a.canon through the warp's shared memory sm.
+struct OutTo {
+    void* sm = nullptr;
+    int lane = 0;
+    bool valid = true;
+};
+
+template <typename T>
+DEV_INLINE void wilson_store_canon(const ApplyArgs& a, const OutTo& w, int v, long s, const cx<typename Store<T>::A>* p)
+{
+    if constexpr (sizeof(T) == 8) {
+        double2 u[12];
+#pragma unroll
+        for (int i = 0; i < 12; ++i) u[i] = unit1(p[i]);
+        warp_store<12>(static_cast<double2*>(w.sm), static_cast<double2*>(a.canon), (size_t)a.Nv * 12, (size_t)v * 12,
+                       (int)s, w.valid, w.lane, u);
+    } else {
+        float4 u[6];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) u[i] = unit2(p[2 * i], p[2 * i + 1]);
+        warp_store<6>(static_cast<float4*>(w.sm), static_cast<float4*>(a.canon), (size_t)a.Nv * 6, (size_t)v * 6, (int)s,
+                      w.valid, w.lane, u);
+    }
+}
+// the R staggered right-hand sides from v0 on: a run of 3 R complex numbers, or what is left of them
+template <typename T, int R>
+DEV_INLINE void staggered_store_canon(const ApplyArgs& a, const OutTo& w, int v0, long s,
+                                      const cx<typename Store<T>::A> (&p)[R][3])
+{
+    using U = typename Store<T>::One;
+    U* sm = static_cast<U*>(w.sm);
+    U* dst = static_cast<U*>(a.canon);
+    if (v0 + R <= a.Nv) {
+        U u[3 * R];
+#pragma unroll
+        for (int i = 0; i < 3 * R; ++i) u[i] = unit1(p[i / 3][i % 3]);
+        warp_store<3 * R>(sm, dst, (size_t)a.Nv * 3, (size_t)v0 * 3, (int)s, w.valid, w.lane, u);
+    } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            if (v0 + r >= a.Nv) break;
+            U u[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) u[i] = unit1(p[r][i]);
+            warp_store<3>(sm, dst, (size_t)a.Nv * 3, (size_t)(v0 + r) * 3, (int)s, w.valid, w.lane, u);
+        }
+    }
 }
 
 // ---------------------------------------------------------------- Wilson
@@ -136,8 +187,8 @@ template <typename A> DEV_INLINE A diag_mode(const ApplyArgs& a, int v, int mode
     return diag_of<A>(a, v);
 }
 
-template <typename T, int R, bool DAG, int MODE = 0, int LF = 0>
-DEV_INLINE void wilson_site(const ApplyArgs& a, long s, int group)
+template <typename T, int R, bool DAG, int MODE = 0, int LF = 0, bool CANON = false>
+DEV_INLINE void wilson_site(const ApplyArgs& a, long s, int group, OutTo to = OutTo())
 {
     constexpr bool FULL = MODE != 0;
     using A = typename Store<T>::A;
@@ -175,7 +226,10 @@ DEV_INLINE void wilson_site(const ApplyArgs& a, long s, int group)
             o.im = fma(mh, acc[r][i].im, dg * p[i].im);
             p[i] = o;
         }
-        if (FULL || v0 + r < a.Nv) store_spinor<T, 12>(a.out, a.g.vol, v0 + r, s, p);
+        if (FULL || v0 + r < a.Nv) {
+            if constexpr (CANON) wilson_store_canon<T>(a, to, v0 + r, s, p);
+            else store_spinor<T, 12>(a.out, a.g.vol, v0 + r, s, p);
+        }
     }
 }
 
@@ -192,8 +246,8 @@ DEV_INLINE void wilson_site(const ApplyArgs& a, long s, int group)
 // lane: the thread's lane in its warp; the warp's 32 consecutive work items
 // start at a multiple of 32, so lane = x mod Lx and the row occupies the lanes
 // lane - x .. lane - x + Lx - 1
-template <typename T, int R, bool DAG, int MODE = 0, int LF = 0>
-DEV_INLINE void wilson_site_xlast(const ApplyArgs& a, long s, int lane, int group)
+template <typename T, int R, bool DAG, int MODE = 0, int LF = 0, bool CANON = false>
+DEV_INLINE void wilson_site_xlast(const ApplyArgs& a, long s, int lane, int group, OutTo to = OutTo())
 {
     constexpr bool FULL = MODE != 0;
     using A = typename Store<T>::A;
@@ -245,7 +299,10 @@ DEV_INLINE void wilson_site_xlast(const ApplyArgs& a, long s, int lane, int grou
             o.im = fma(mh, acc[r][i].im, dg * pc[i].im);
             pc[i] = o;
         }
-        if (FULL || v0 + r < a.Nv) store_spinor<T, 12>(a.out, a.g.vol, v0 + r, s, pc);
+        if (FULL || v0 + r < a.Nv) {
+            if constexpr (CANON) wilson_store_canon<T>(a, to, v0 + r, s, pc);
+            else store_spinor<T, 12>(a.out, a.g.vol, v0 + r, s, pc);
+        }
     }
 }
 
@@ -623,9 +680,42 @@ DEV_INLINE void wilson_site_pipe(const ApplyArgs& a, long s, int group, char* sm
 }
 
 // ---------------------------------------------------------------- staggered
-// MODE and LF as in wilson_site
-template <typename T, int R, bool DAG, int MODE = 0, int LF = 0>
-DEV_INLINE void staggered_site(const ApplyArgs& a, long s, int group)
+// acc += eta (Uf pf - Ub^+ pb), the sign eta in bit 31.  FP32: the two hops of a
+// direction are summed before they join the others (a chain of all 24 products
+// of a component rounds half again as much).  FP64 and double-float: eta is a
+// sign flip of the spinors and the products go straight into the sums.
+template <typename A>
+DEV_INLINE void staggered_hops(const cx<A>* Uf, const cx<A>* Ub, cx<A>* pf, cx<A>* pb, uint32_t eta, cx<A>* acc)
+{
+    const uint32_t m = eta & 0x80000000u;
+    if constexpr (std::is_same<A, float>::value) {
+        const float e = m ? -1.f : 1.f;
+        cx<A> w[3], wb[3];
+        mat_vec(Uf, pf, w);
+        mat_dag_vec(Ub, pb, wb);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const cx<A> d = w[c] - wb[c];
+            acc[c].re = fma(e, d.re, acc[c].re);
+            acc[c].im = fma(e, d.im, acc[c].im);
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            pf[c] = cx<A>{flip_sign(pf[c].re, m), flip_sign(pf[c].im, m)};
+            pb[c] = cx<A>{flip_sign(pb[c].re, m ^ 0x80000000u), flip_sign(pb[c].im, m ^ 0x80000000u)};
+        }
+        mat_vec_acc(Uf, pf, acc);
+        mat_dag_vec_acc(Ub, pb, acc);
+    }
+}
+
+// MODE and LF as in wilson_site.  FP64: 288 multiply-adds and 12 operations for
+// the diagonal (348 operations with the hops summed by themselves) per site and
+// right-hand side, which is what bounds the sweep (16^4, Nv = 8: 322 -> 272 us, 0.59 T
+// operations per second).
+template <typename T, int R, bool DAG, int MODE = 0, int LF = 0, bool CANON = false>
+DEV_INLINE void staggered_site(const ApplyArgs& a, long s, int group, OutTo to = OutTo())
 {
     constexpr bool FAST = MODE != 0;
     using A = typename Store<T>::A;
@@ -641,7 +731,7 @@ DEV_INLINE void staggered_site(const ApplyArgs& a, long s, int group)
     int par = 0;  // x_0 + ... + x_{mu-1}
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
-        const A eta = (par & 1) ? A(-1) : A(1);
+        const uint32_t eta = (uint32_t)par << 31;
         par += x[mu];
         cx<A> Uf[9], Ub[9];
         load_link_f<T, false, LF>(a.links, a.g.vol, mu, s, Uf);
@@ -649,17 +739,10 @@ DEV_INLINE void staggered_site(const ApplyArgs& a, long s, int group)
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int v = FAST ? v0 + r : min(v0 + r, a.Nv - 1);   // partial group: recompute, store guarded
-            cx<A> pf[3], pb[3], w[3] = {}, wb[3] = {};
+            cx<A> pf[3], pb[3];
             load_spinor<T, 3>(a.in, a.g.vol, v, s + fwd[mu], pf);
             load_spinor<T, 3>(a.in, a.g.vol, v, s + bwd[mu], pb);
-            mat_vec(Uf, pf, w);
-            mat_dag_vec(Ub, pb, wb);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                cx<A> d = w[c] - wb[c];
-                acc[r][c].re = fma(eta, d.re, acc[r][c].re);
-                acc[r][c].im = fma(eta, d.im, acc[r][c].im);
-            }
+            staggered_hops(Uf, Ub, pf, pb, mu == 0 ? 0u : eta, acc[r]);
         }
     }
     const A hf = DAG ? A(-0.5) : A(0.5);
@@ -676,16 +759,20 @@ DEV_INLINE void staggered_site(const ApplyArgs& a, long s, int group)
             o.im = fma(hf, acc[r][c].im, dg * p[c].im);
             p[c] = o;
         }
-        if (FAST || v0 + r < a.Nv) store_spinor<T, 3>(a.out, a.g.vol, v0 + r, s, p);
+        if constexpr (CANON) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) acc[r][c] = p[c];
+        } else if (FAST || v0 + r < a.Nv) store_spinor<T, 3>(a.out, a.g.vol, v0 + r, s, p);
     }
+    if constexpr (CANON) staggered_store_canon<T, R>(a, to, v0, s, acc);
 }
 
 // staggered_site with the x hops last, by lane exchange of the site's own
 // spinor (the warp layout of wilson_site_xlast: whole x-rows per warp, lane
 // the thread's lane): lane x sends psi(x) to lane x - 1 for its forward hop
 // and V_x(x)^+ psi(x) to lane x + 1 for its backward hop (eta_0 = 1)
-template <typename T, int R, bool DAG, int MODE = 0, int LF = 0>
-DEV_INLINE void staggered_site_xlast(const ApplyArgs& a, long s, int lane, int group)
+template <typename T, int R, bool DAG, int MODE = 0, int LF = 0, bool CANON = false>
+DEV_INLINE void staggered_site_xlast(const ApplyArgs& a, long s, int lane, int group, OutTo to = OutTo())
 {
     constexpr bool FAST = MODE != 0;
     using A = typename Store<T>::A;
@@ -704,7 +791,7 @@ DEV_INLINE void staggered_site_xlast(const ApplyArgs& a, long s, int lane, int g
     int par = x[0];  // x_0 + ... + x_{mu-1}, from mu = 1 on
 #pragma unroll
     for (int mu = 1; mu < 4; ++mu) {
-        const A eta = (par & 1) ? A(-1) : A(1);
+        const uint32_t eta = (uint32_t)par << 31;
         par += x[mu];
         cx<A> Uf[9], Ub[9];
         load_link_f<T, false, LF>(a.links, a.g.vol, mu, s, Uf);
@@ -712,17 +799,10 @@ DEV_INLINE void staggered_site_xlast(const ApplyArgs& a, long s, int lane, int g
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int v = FAST ? v0 + r : min(v0 + r, a.Nv - 1);
-            cx<A> pf[3], pb[3], w[3] = {}, wb[3] = {};
+            cx<A> pf[3], pb[3];
             load_spinor<T, 3>(a.in, a.g.vol, v, s + fwd[mu], pf);
             load_spinor<T, 3>(a.in, a.g.vol, v, s + bwd[mu], pb);
-            mat_vec(Uf, pf, w);
-            mat_dag_vec(Ub, pb, wb);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                cx<A> d = w[c] - wb[c];
-                acc[r][c].re = fma(eta, d.re, acc[r][c].re);
-                acc[r][c].im = fma(eta, d.im, acc[r][c].im);
-            }
+            staggered_hops(Uf, Ub, pf, pb, mu == 0 ? 0u : eta, acc[r]);
         }
     }
     cx<A> U[9];
@@ -751,8 +831,12 @@ DEV_INLINE void staggered_site_xlast(const ApplyArgs& a, long s, int lane, int g
             o.im = fma(hf, t.im, dg * p[c].im);
             p[c] = o;
         }
-        if (FAST || v0 + r < a.Nv) store_spinor<T, 3>(a.out, a.g.vol, v0 + r, s, p);
+        if constexpr (CANON) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) acc[r][c] = p[c];
+        } else if (FAST || v0 + r < a.Nv) store_spinor<T, 3>(a.out, a.g.vol, v0 + r, s, p);
     }
+    if constexpr (CANON) staggered_store_canon<T, R>(a, to, v0, s, acc);
 }
 
 // ---------------------------------------------------------------- Brillouin

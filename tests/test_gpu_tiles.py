@@ -45,3 +45,37 @@ def test_brillouin_tensor_core_tiles(dg, L, Nv, prec):
             want = oracle.apply("brillouin", V, psi, 0.05, dagger=dag)
             assert rel_l2(got, want) <= TOL[prec], (order, dag)
     D.close()
+
+
+# whole and partial warps of sites, partial groups of right-hand sides, one and several blocks
+@pytest.mark.parametrize("op", ["wilson", "staggered"])
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+@pytest.mark.parametrize("L,Nv", [((3, 2, 5, 2), 1), ((7, 5, 3, 3), 5), ((8, 4, 4, 2), 8), ((16, 4, 2, 4), 7)])
+def test_canonical_output_is_the_internal_one(dg, op, prec, L, Nv):
+    """A sweep that writes a canonical field itself stores the numbers that
+    unpacking its internal result gives, in every launch shape, and leaves no
+    entry out; backward gives what apply_dagger and force give."""
+    cdt = torch.complex128 if prec == "f64" else torch.complex64
+    V = torch.from_numpy(synth.gauge_links(L, 3, "near_identity", 61)).to(cdt).cuda()
+    x = torch.from_numpy(synth.spinor(L, Nv, NS[op], 3, 62)).to(cdt).cuda()
+    g = torch.from_numpy(synth.spinor(L, Nv, NS[op], 3, 63)).to(cdt).cuda()
+    D = dg.Dirac(op, L, Nv, 0.12, prec)
+    D.set_links(V)
+    done = 0
+    for R in (1, 2, 4, 6):
+        for block in (32, 64, 128, 256):
+            for variant in (0, 1, 6):
+                if not dg.config_supported(op, prec, R, block, variant, L):
+                    continue
+                D.set_kernel_config(R, block, variant)
+                done += 1
+                for dag in (False, True):
+                    want = D.unpack(D.apply(D.pack(x), dagger=dag))
+                    got = D.new_canonical()
+                    got.fill_(complex(float("nan"), float("nan")))
+                    D.apply(x, out=got, dagger=dag)
+                    assert torch.equal(torch.view_as_real(got), torch.view_as_real(want)), (R, block, variant, dag)
+    assert done >= 4
+    gpsi, F = D.backward(x, g)
+    assert torch.equal(gpsi, D.apply_dagger(g)) and torch.equal(F, D.force(x, g))
+    D.close()
