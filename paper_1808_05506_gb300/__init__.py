@@ -135,19 +135,32 @@ def check(status: int, h=None, what: str = "") -> None:
         raise DiracError(status, f"{what}: {last_error(h)}")
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
-def _stream_ptr(stream=None):
+# The smallest sweeps take 5 us on the GPU, so what the binding does per call
+# decides their rate: the stream handle without a Stream object, pointers as the
+# plain integers ctypes takes for void*, and sizes asked of the library once.
+def _stream_ptr(stream=None) -> int:
+    if stream is not None:
+        return stream.cuda_stream
     torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
-def _ptr(t) -> ctypes.c_void_p:
-    return ctypes.c_void_p(t.data_ptr())
+def _ptr(t) -> int:
+    return t.data_ptr()
 
 
 def _is_device(t) -> bool:
@@ -205,9 +218,16 @@ class Dirac:
         check(lib().dirac_field_bytes(self.h, layout, ctypes.byref(n)), self.h, "dirac_field_bytes")
         return n.value
 
+    def _internal_bytes(self) -> int:
+        """field_bytes(INTERNAL), which does not change over the handle's life."""
+        n = self.__dict__.get("_nbytes")
+        if n is None:
+            n = self._nbytes = self.field_bytes(INTERNAL)
+        return n
+
     def new_internal(self):
         torch = _torch()
-        return torch.empty(self.field_bytes(INTERNAL), dtype=torch.uint8, device=self.device)
+        return torch.empty(self._internal_bytes(), dtype=torch.uint8, device=self.device)
 
     def new_canonical(self):
         torch = _torch()
@@ -245,13 +265,15 @@ class Dirac:
     def _internal(self, t, what="internal field"):
         torch = _torch()
         if t.dtype != torch.uint8 or not _is_device(t) or not t.is_contiguous() \
-                or t.numel() < self.field_bytes(INTERNAL):
+                or t.numel() < self._internal_bytes():
             raise ValueError(f"{what} must be a contiguous CUDA uint8 buffer of at least "
-                             f"{self.field_bytes(INTERNAL)} bytes (new_internal)")
+                             f"{self._internal_bytes()} bytes (new_internal)")
         return t
 
     def _sync_stream(self):
-        check(lib().dirac_set_stream(self.h, _stream_ptr(self._stream)), self.h, "dirac_set_stream")
+        st = lib().dirac_set_stream(self.h, _stream_ptr(self._stream))
+        if st != OK:
+            check(st, self.h, "dirac_set_stream")
 
     # -- calls ------------------------------------------------------------------
     def set_links(self, V, remember: bool = True):
@@ -325,8 +347,9 @@ class Dirac:
             out = self.new_canonical() if out is None else self._canon_out(out)
         self._sync_stream()
         fn = lib().dirac_apply_dagger if dagger else lib().dirac_apply
-        check(fn(self.h, _ptr(out), _ptr(x), layout),
-              self.h, "dirac_apply_dagger" if dagger else "dirac_apply")
+        st = fn(self.h, _ptr(out), _ptr(x), layout)
+        if st != OK:
+            check(st, self.h, "dirac_apply_dagger" if dagger else "dirac_apply")
         return out
 
     def apply_host(self, x, out=None, dagger: bool = False, sync: bool = True):
