@@ -240,7 +240,7 @@ dirac_status dirac_create(dirac_handle** h, dirac_op op, int Nc, int Nx, int Ny,
         delete H;
         return DIRAC_ERR_CUDA;
     }
-    H->cfg = default_config(H->op, H->prec, Nv);
+    H->cfg = default_config(H->op, H->prec, Nv, &H->g);
     if (cudaMalloc((void**)&H->dev_err, sizeof(int)) != cudaSuccess || cudaMemset(H->dev_err, 0, sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         g_create_error = "dirac_create: cannot allocate the device error word";
@@ -778,18 +778,51 @@ bool apply_config_supported(int op, int prec, int R, int block, int variant, con
     return op == OP_WILSON && variant == V_PIPE3 && wilson_pipe_smem(prec, R, block, 3) <= 227 * 1024;
 }
 
-LaunchCfg default_config(int op, int prec, int Nv)
+// The launch shape of a handle that was not tuned.  Wilson and staggered sweeps of
+// FP32 and 16-bit storage are bound by what they read through L2, so the shapes
+// that read least come first: x hops last by lane exchange (variant 6) where
+// the lattice allows it, else the groups of a site in one block (variant 1).
+// Right-hand sides per thread R: the largest that leaves little of the last
+// block's groups empty.  Lexicographic order, except where a t-slice and
+// its result take more than 25 MB, a good part of the L2 (then t-chunks).
+// Measured against variant 0, R dividing Nv, 128 threads (FP32, us):
+//   Wilson 16^3x32 Nv = 12 109 -> 94, 32x16^3 Nv = 8 76 -> 65, 32^4 Nv = 12
+//   1010 -> 777, 24^4 Nv = 12 297 -> 253, 20x18x16x24 Nv = 5 64 -> 62;
+//   staggered 16^3x32 Nv = 12 51 -> 39, 32^4 Nv = 4 130 -> 101, Nv = 3 148 -> 108,
+//   24^4 Nv = 12 114 -> 95, 16x18x20x32 Nv = 24 122 -> 101.
+// FP64 and Brillouin sweeps are bound by arithmetic: variant 0.
+LaunchCfg default_config(int op, int prec, int Nv, const Geom* g)
 {
-    // the largest right-hand-side group that divides Nv and fits the
-    // registers without spilling (FP64 sweeps use at most 2 / 4)
-    if (op == OP_STAGGERED) {
-        int R = (Nv % 6 == 0) ? 6 : (Nv % 4 == 0 ? 4 : (Nv % 2 == 0 ? 2 : 1));
-        if (prec == P_F64 && R > 4) R = 4;
-        return LaunchCfg{R, 128, V_DIRECT};
+    if (op == OP_BRILLOUIN || prec == P_F64 || !g) {
+        if (op == OP_STAGGERED) {
+            int R = (Nv % 6 == 0) ? 6 : (Nv % 4 == 0 ? 4 : (Nv % 2 == 0 ? 2 : 1));
+            if (prec == P_F64 && R > 4) R = 4;
+            return LaunchCfg{R, 128, V_DIRECT};
+        }
+        return LaunchCfg{(Nv % 2 == 0) ? 2 : 1, 128, V_DIRECT};
     }
-    if (prec == P_F64) return LaunchCfg{(Nv % 2 == 0) ? 2 : 1, 128, V_DIRECT};
-    int R = (Nv % 2 == 0) ? 2 : 1;
-    return LaunchCfg{R, 128, V_DIRECT};
+    const bool xlast = 32 % g->L[0] == 0 && g->stride[3] % 32 == 0;
+    const int block = xlast ? 32 : 64;
+    const double slice = (double)g->stride[3] * Nv * nsc_of(op) * cbytes(prec);
+    const int order = slice > 25e6 ? (g->L[3] < 8 ? g->L[3] : 8) : 0;
+    int R = 1;
+    if (op == OP_WILSON) {
+        R = (Nv % 2 == 0 || Nv >= 5) ? 2 : 1;
+    } else {
+        // right-hand sides the blocks compute, times what a thread of few costs more
+        double best = 0.0;
+        const int Rs[] = {6, 4, 2, 1};
+        const double f[] = {xlast ? 1.05 : 1.0, 1.0, 1.1, 1.5};
+        for (int i = 0; i < 4; ++i) {
+            const int ng = (Nv + Rs[i] - 1) / Rs[i], gy = groups_per_block(block, ng);
+            const double cost = (double)((ng + gy - 1) / gy * gy) * Rs[i] * f[i];
+            if (best == 0.0 || cost < best) {
+                best = cost;
+                R = Rs[i];
+            }
+        }
+    }
+    return LaunchCfg{R, block, xlast ? V_XLAST : V_GROUPS, order};
 }
 
 cudaError_t launch_apply(int op, int prec, bool dagger, const ApplyArgs& a, LaunchCfg cfg, cudaStream_t st)

@@ -7,7 +7,7 @@
 #include "dirac_internal.h"
 
 namespace dirac {
-LaunchCfg default_config(int op, int prec, int Nv);
+LaunchCfg default_config(int op, int prec, int Nv, const Geom* g = nullptr);   // g: of the handle's sweeps
 }
 
 struct dirac_handle {

@@ -79,3 +79,23 @@ def test_canonical_output_is_the_internal_one(dg, op, prec, L, Nv):
     gpsi, F = D.backward(x, g)
     assert torch.equal(gpsi, D.apply_dagger(g)) and torch.equal(F, D.force(x, g))
     D.close()
+
+
+# the launch shapes of handles that were not tuned: x-rows in a warp or not, R by Nv, t-chunks or not
+@pytest.mark.parametrize("op", ["wilson", "staggered"])
+@pytest.mark.parametrize("prec", ["f32", "bf16"])
+@pytest.mark.parametrize("L,Nv", [((8, 4, 2, 3), 1), ((8, 4, 2, 3), 5), ((6, 3, 2, 5), 3), ((5, 3, 3, 2), 7),
+                                  ((4, 4, 2, 2), 12), ((3, 2, 2, 3), 24)])
+def test_default_launch_shape(dg, op, prec, L, Nv):
+    V = synth.round_to(synth.gauge_links(L, 3, "near_identity", 71), "f32")
+    psi = synth.round_to(synth.spinor(L, Nv, NS[op], 3, 72), prec)
+    mass = 0.12
+    D = dg.Dirac(op, L, Nv, mass, prec)
+    D.set_links(torch.from_numpy(V).cuda())
+    Vs = synth.round_to(V, prec)
+    x = torch.from_numpy(psi.astype(np.complex64)).cuda()
+    m0 = oracle.kappa_to_m0(mass) if op == "wilson" else mass
+    for dag in (False, True):
+        got = D.apply(x, dagger=dag).cpu().numpy().astype(np.complex128)
+        assert rel_l2(got, oracle.apply(op, Vs, psi, m0, dagger=dag)) <= TOL[prec]
+    D.close()
