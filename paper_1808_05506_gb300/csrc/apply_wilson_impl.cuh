@@ -92,7 +92,8 @@ __global__ void __launch_bounds__(192, 2) k_wilson_groups(ApplyArgs a, int ngrou
         wilson_site<T, R, DAG, MODE, LF, true>(a, slab_site(a, min(p, a.nsites - 1)), group, to);
     } else {
         if (p >= a.nsites || group >= ngroups) return;
-        wilson_site<T, R, DAG, MODE, LF>(a, slab_site(a, p), group);
+        if constexpr (R == 2 && sizeof(T) == 2) wilson_site2<T, DAG, MODE, LF, false>(a, slab_site(a, p), 0, group);
+        else wilson_site<T, R, DAG, MODE, LF>(a, slab_site(a, p), group);
     }
 }
 
@@ -111,7 +112,8 @@ __global__ void __launch_bounds__(192, 2) k_wilson_xlast(ApplyArgs a, int ngroup
         const OutTo to{sm[(threadIdx.y * blockDim.x + threadIdx.x) >> 5], (int)(threadIdx.x & 31), true};
         wilson_site_xlast<T, R, DAG, MODE, LF, true>(a, slab_site(a, p), threadIdx.x & 31, group, to);
     } else {
-        wilson_site_xlast<T, R, DAG, MODE, LF>(a, slab_site(a, p), threadIdx.x & 31, group);
+        if constexpr (R == 2 && sizeof(T) == 2) wilson_site2<T, DAG, MODE, LF, true>(a, slab_site(a, p), threadIdx.x & 31, group);
+        else wilson_site_xlast<T, R, DAG, MODE, LF>(a, slab_site(a, p), threadIdx.x & 31, group);
     }
 }
 

@@ -465,6 +465,28 @@ DEV_INLINE f2 ffma2(f2 a, f2 b, f2 c)
     return f2{fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y)};
 #endif
 }
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
+#define DIRAC_F2_OP(name, op)                                               \
+    DEV_INLINE f2 name(f2 a, f2 b)                                          \
+    {                                                                       \
+        unsigned long long ra, rb, rd;                                      \
+        asm("mov.b64 %0, {%1, %2};" : "=l"(ra) : "f"(a.x), "f"(a.y));       \
+        asm("mov.b64 %0, {%1, %2};" : "=l"(rb) : "f"(b.x), "f"(b.y));       \
+        asm(op " %0, %1, %2;" : "=l"(rd) : "l"(ra), "l"(rb));               \
+        f2 d;                                                               \
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(rd));      \
+        return d;                                                           \
+    }
+DIRAC_F2_OP(fadd2, "add.rn.f32x2")
+DIRAC_F2_OP(fsub2, "sub.rn.f32x2")
+DIRAC_F2_OP(fmul2, "mul.rn.f32x2")
+#undef DIRAC_F2_OP
+#else
+DEV_INLINE f2 fadd2(f2 a, f2 b) { return f2{a.x + b.x, a.y + b.y}; }
+DEV_INLINE f2 fsub2(f2 a, f2 b) { return f2{a.x - b.x, a.y - b.y}; }
+DEV_INLINE f2 fmul2(f2 a, f2 b) { return f2{a.x * b.x, a.y * b.y}; }
+#endif
+
 // acc += s * u  (s real)
 DEV_INLINE cx<float> caxpy2(float s, cx<float> u, cx<float> acc)
 {

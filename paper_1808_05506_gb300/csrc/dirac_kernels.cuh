@@ -306,6 +306,288 @@ DEV_INLINE void wilson_site_xlast(const ApplyArgs& a, long s, int lane, int grou
     }
 }
 
+// ---------------------------------------------------------------- Wilson, pairs of right-hand sides
+// The sweeps of two right-hand sides per thread of 16-bit fields, with the two in
+// the halves of packed FP32 registers: one f32x2 instruction does both, each link entry
+// is broadcast once for 2 x 2 colour vectors, and the spin projections, done right-hand side
+// by right-hand side, write their halves without moves (pairs of (re, im), tried
+// before, needed a swapped copy of every factor).  A quarter of the sweep's
+// instructions go, and 16-bit sweeps, which also unpack every value, gain by it:
+// 16^3 x 32, Nv = 24, BF16, variant 6: 208 -> 169 us, with the loads one hop ahead 166 (the best shape
+// before, variant 5: 187); 32^4, Nv = 12: 656 (variant 5: 718).  FP32 sweeps keep the
+// scalar form: at 12 warps per SM they wait for memory whatever they execute (32^4,
+// Nv = 12: 131 -> 97 M instructions, 0.70 -> 0.73 ms, and the same with loads ahead).
+struct c2 { f2 re, im; };   // a complex number of each right-hand side
+
+DEV_INLINE void set_half(c2& p, int r, cx<float> v)
+{
+    if (r == 0) { p.re.x = v.re; p.im.x = v.im; }
+    else { p.re.y = v.re; p.im.y = v.im; }
+}
+
+// colour a of w = U h (or U^+ h) for the two half-spinor components
+template <bool BACK>
+DEV_INLINE void row2(const cx<float>* U, int a, const c2* h, c2& w0, c2& w1)
+{
+    f2 t0, t1;   // sum of u_im h_im (re part) or u_im h_re (im part of U^+), subtracted at the end
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        const cx<float> u = BACK ? U[3 * b + a] : U[3 * a + b];
+        const f2 ur{u.re, u.re}, ui{u.im, u.im};
+        if (b == 0) {
+            w0.re = fmul2(ur, h[0].re);
+            w1.re = fmul2(ur, h[3].re);
+            w0.im = fmul2(ur, h[0].im);
+            w1.im = fmul2(ur, h[3].im);
+            t0 = fmul2(ui, BACK ? h[0].re : h[0].im);
+            t1 = fmul2(ui, BACK ? h[3].re : h[3].im);
+        } else {
+            w0.re = ffma2(ur, h[b].re, w0.re);
+            w1.re = ffma2(ur, h[3 + b].re, w1.re);
+            w0.im = ffma2(ur, h[b].im, w0.im);
+            w1.im = ffma2(ur, h[3 + b].im, w1.im);
+            t0 = ffma2(ui, BACK ? h[b].re : h[b].im, t0);
+            t1 = ffma2(ui, BACK ? h[3 + b].re : h[3 + b].im, t1);
+        }
+        if (BACK) {
+            w0.re = ffma2(ui, h[b].im, w0.re);
+            w1.re = ffma2(ui, h[3 + b].im, w1.re);
+        } else {
+            w0.im = ffma2(ui, h[b].re, w0.im);
+            w1.im = ffma2(ui, h[3 + b].re, w1.im);
+        }
+    }
+    if (BACK) {
+        w0.im = fsub2(w0.im, t0);
+        w1.im = fsub2(w1.im, t1);
+    } else {
+        w0.re = fsub2(w0.re, t0);
+        w1.re = fsub2(w1.re, t1);
+    }
+}
+
+DEV_INLINE c2 add2(c2 a, c2 b) { return {fadd2(a.re, b.re), fadd2(a.im, b.im)}; }
+DEV_INLINE c2 sub2(c2 a, c2 b) { return {fsub2(a.re, b.re), fsub2(a.im, b.im)}; }
+DEV_INLINE c2 addi2(c2 a, c2 b) { return {fsub2(a.re, b.im), fadd2(a.im, b.re)}; }   // a + i b
+DEV_INLINE c2 subi2(c2 a, c2 b) { return {fadd2(a.re, b.im), fsub2(a.im, b.re)}; }   // a - i b
+
+// wilson_reconstruct of colour c
+template <int MU, int S>
+DEV_INLINE void reconstruct2(int c, c2 w0, c2 w1, c2* acc)
+{
+    acc[c] = add2(acc[c], w0);
+    acc[3 + c] = add2(acc[3 + c], w1);
+    if constexpr (MU == 0) {
+        acc[6 + c] = S > 0 ? addi2(acc[6 + c], w1) : subi2(acc[6 + c], w1);
+        acc[9 + c] = S > 0 ? addi2(acc[9 + c], w0) : subi2(acc[9 + c], w0);
+    } else if constexpr (MU == 1) {
+        acc[6 + c] = S > 0 ? add2(acc[6 + c], w1) : sub2(acc[6 + c], w1);
+        acc[9 + c] = S > 0 ? sub2(acc[9 + c], w0) : add2(acc[9 + c], w0);
+    } else if constexpr (MU == 2) {
+        acc[6 + c] = S > 0 ? addi2(acc[6 + c], w0) : subi2(acc[6 + c], w0);
+        acc[9 + c] = S > 0 ? subi2(acc[9 + c], w1) : addi2(acc[9 + c], w1);
+    } else {
+        acc[6 + c] = S > 0 ? add2(acc[6 + c], w0) : sub2(acc[6 + c], w0);
+        acc[9 + c] = S > 0 ? add2(acc[9 + c], w1) : sub2(acc[9 + c], w1);
+    }
+}
+
+// The spinors of two right-hand sides at one site, and a link, as loaded.  The loads
+// are volatile: they are issued where they stand, one hop ahead of their use
+// (the compiler, short of registers, would sink them to it).
+template <typename T> struct Raw2 {
+    static constexpr int K = SpinorLayout<T, 12>::K;
+    uint4 e[2][K];
+};
+DEV_INLINE uint4 ld_now(const uint4* p)
+{
+#if defined(__CUDA_ARCH__)
+    uint4 v;
+    asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+#else
+    return *p;
+#endif
+}
+DEV_INLINE uint32_t ld_now(const uint32_t* p)
+{
+#if defined(__CUDA_ARCH__)
+    uint32_t v;
+    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+#else
+    return *p;
+#endif
+}
+template <typename T, bool FULL>
+DEV_INLINE void raw_load(const ApplyArgs& a, int v0, long s, Raw2<T>& p)
+{
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int v = FULL ? v0 + r : min(v0 + r, a.Nv - 1);
+        const uint4* q = static_cast<const uint4*>(a.in) + blk_index(a.g.vol, Raw2<T>::K, v, 0, s);
+#pragma unroll
+        for (int k = 0; k < Raw2<T>::K; ++k) p.e[r][k] = ld_now(q + 32 * k);
+    }
+}
+template <typename T> DEV_INLINE void raw_spinor(const Raw2<T>& p, int r, cx<float>* o)
+{
+#pragma unroll
+    for (int k = 0; k < Raw2<T>::K; ++k) {
+        const uint4 v = p.e[r][k];
+        o[4 * k] = unpack2(v.x, (T*)nullptr);
+        o[4 * k + 1] = unpack2(v.y, (T*)nullptr);
+        o[4 * k + 2] = unpack2(v.z, (T*)nullptr);
+        o[4 * k + 3] = unpack2(v.w, (T*)nullptr);
+    }
+}
+template <typename T, int LF> struct RawLink {
+    static constexpr int N = LF == 1 ? 6 : 9;
+    uint32_t e[N];
+};
+template <typename T, int LF>
+DEV_INLINE void raw_link(const ApplyArgs& a, int mu, long s, RawLink<T, LF>& u)
+{
+    const uint32_t* q = static_cast<const uint32_t*>(a.links) + blk_index(a.g.vol, RawLink<T, LF>::N, mu, 0, s);
+#pragma unroll
+    for (int e = 0; e < RawLink<T, LF>::N; ++e) u.e[e] = ld_now(q + 32 * e);
+}
+template <typename T, int LF> DEV_INLINE void link_of(const RawLink<T, LF>& u, cx<float>* U)
+{
+#pragma unroll
+    for (int e = 0; e < RawLink<T, LF>::N; ++e) U[e] = unpack2(u.e[e], (T*)nullptr);
+    if constexpr (LF == 1) reconstruct_row2(U);
+}
+
+DEV_INLINE c2 shfl2(c2 v, int src)
+{
+#if defined(__CUDA_ARCH__)
+    return {{__shfl_sync(0xffffffffu, v.re.x, src), __shfl_sync(0xffffffffu, v.re.y, src)},
+            {__shfl_sync(0xffffffffu, v.im.x, src), __shfl_sync(0xffffffffu, v.im.y, src)}};
+#else
+    (void)src;
+    return v;
+#endif
+}
+
+// hop number H of wilson_site2: x (not XL), y, z, t, forward and backward
+template <int H, bool XL> struct Hop2 {
+    static constexpr int MU = H / 2 + (XL ? 1 : 0);
+    static constexpr bool BACK = (H & 1) != 0;
+};
+template <typename T, int H, int NH, bool DAG, bool FULL, int LF, bool XL>
+DEV_INLINE void wilson_hops2(const ApplyArgs& a, long s, const long* fwd, const long* bwd, int v0, Raw2<T>& p,
+                             RawLink<T, LF>& u, c2 (&acc)[12])
+{
+    using Q = Hop2<H, XL>;
+    constexpr int S = (DAG != Q::BACK) ? +1 : -1;
+    c2 h[6];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        cx<float> ps[12], g[6];
+        raw_spinor<T>(p, r, ps);
+        wilson_project<Q::MU, S>(ps, g);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) set_half(h[i], r, g[i]);
+    }
+    // the next hop's spinors and link, or the site's own and its x link
+    RawLink<T, LF> un;
+    if constexpr (H + 1 < NH) {
+        using N = Hop2<H + 1, XL>;
+        const long nb = s + (N::BACK ? bwd[N::MU] : fwd[N::MU]);
+        raw_load<T, FULL>(a, v0, nb, p);
+        raw_link<T, LF>(a, N::MU, N::BACK ? nb : s, un);
+    } else {
+        raw_load<T, FULL>(a, v0, s, p);
+        if constexpr (XL) raw_link<T, LF>(a, 0, s, un);
+    }
+    cx<float> U[9];
+    link_of<T, LF>(u, U);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        c2 w0, w1;
+        row2<Q::BACK>(U, c, h, w0, w1);
+        reconstruct2<Q::MU, S>(c, w0, w1, acc);
+    }
+    if constexpr (H + 1 < NH || XL) u = un;
+    if constexpr (H + 1 < NH) wilson_hops2<T, H + 1, NH, DAG, FULL, LF, XL>(a, s, fwd, bwd, v0, p, u, acc);
+}
+
+// wilson_site (XL = false) and wilson_site_xlast (XL = true) for two right-hand sides
+template <typename T, bool DAG, int MODE, int LF, bool XL>
+DEV_INLINE void wilson_site2(const ApplyArgs& a, long s, int lane, int group)
+{
+    constexpr bool FULL = MODE != 0;
+    long fwd[4], bwd[4];
+    int x[4];
+    site_offsets(a.g, s, fwd, bwd, x);
+    const int v0 = group * 2;
+    c2 acc[12];
+#pragma unroll
+    for (int i = 0; i < 12; ++i) acc[i] = c2{{0.f, 0.f}, {0.f, 0.f}};
+    constexpr int SF = DAG ? +1 : -1;
+    constexpr int SB = -SF;
+    Raw2<T> p;
+    RawLink<T, LF> u;
+    constexpr int M0 = XL ? 1 : 0;
+    raw_load<T, FULL>(a, v0, s + fwd[M0], p);
+    raw_link<T, LF>(a, M0, s, u);
+    wilson_hops2<T, 0, XL ? 6 : 8, DAG, FULL, LF, XL>(a, s, fwd, bwd, v0, p, u, acc);
+    c2 hf[6], hb[6];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int v = FULL ? v0 + r : min(v0 + r, a.Nv - 1);
+        const float dg = -2.f * diag_mode<float>(a, v, MODE);   // out = -1/2 (acc - 2 diag psi)
+        cx<float> q[12], g[6];
+        raw_spinor<T>(p, r, q);
+#pragma unroll
+        for (int i = 0; i < 12; ++i) {
+            if (r == 0) {
+                acc[i].re.x = fmaf(dg, q[i].re, acc[i].re.x);
+                acc[i].im.x = fmaf(dg, q[i].im, acc[i].im.x);
+            } else {
+                acc[i].re.y = fmaf(dg, q[i].re, acc[i].re.y);
+                acc[i].im.y = fmaf(dg, q[i].im, acc[i].im.y);
+            }
+        }
+        if constexpr (XL) {
+            wilson_project<0, SF>(q, g);
+#pragma unroll
+            for (int i = 0; i < 6; ++i) set_half(hf[i], r, g[i]);
+            wilson_project<0, SB>(q, g);
+#pragma unroll
+            for (int i = 0; i < 6; ++i) set_half(hb[i], r, g[i]);
+        }
+    }
+    if constexpr (XL) {
+        const int Lx = a.g.L[0];
+        const int lane_f = lane - x[0] + (x[0] + 1 == Lx ? 0 : x[0] + 1);   // site x + 1
+        const int lane_b = lane - x[0] + (x[0] == 0 ? Lx - 1 : x[0] - 1);   // site x - 1
+        cx<float> U[9];
+        link_of<T, LF>(u, U);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) hf[i] = shfl2(hf[i], lane_f);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            c2 w0, w1;
+            row2<false>(U, c, hf, w0, w1);
+            reconstruct2<0, SF>(c, w0, w1, acc);
+            row2<true>(U, c, hb, w0, w1);
+            w0 = shfl2(w0, lane_b);
+            w1 = shfl2(w1, lane_b);
+            reconstruct2<0, SB>(c, w0, w1, acc);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        cx<float> o[12];
+#pragma unroll
+        for (int i = 0; i < 12; ++i)
+            o[i] = r == 0 ? cx<float>{-0.5f * acc[i].re.x, -0.5f * acc[i].im.x} : cx<float>{-0.5f * acc[i].re.y, -0.5f * acc[i].im.y};
+        if (FULL || v0 + r < a.Nv) store_spinor<T, 12>(a.out, a.g.vol, v0 + r, s, o);
+    }
+}
+
 // ---------------------------------------------------------------- Wilson, t-march
 // One thread owns the site column (x, y, z) for the slices t0 <= t < t1 and
 // one group of R right-hand sides.  Along t each spinor and each t-link is

@@ -99,3 +99,26 @@ def test_default_launch_shape(dg, op, prec, L, Nv):
         got = D.apply(x, dagger=dag).cpu().numpy().astype(np.complex128)
         assert rel_l2(got, oracle.apply(op, Vs, psi, m0, dagger=dag)) <= TOL[prec]
     D.close()
+
+
+# the packed 16-bit Wilson sweeps: whole and partial pairs, x-rows of 4 to 32 sites and none, both link formats
+@pytest.mark.parametrize("prec", ["bf16", "f16"])
+@pytest.mark.parametrize("L,Nv", [((4, 4, 2, 3), 2), ((32, 2, 2, 2), 3), ((6, 5, 3, 2), 5), ((16, 2, 4, 3), 14)])
+def test_wilson_pairs_16bit(dg, prec, L, Nv):
+    V = synth.round_to(synth.gauge_links(L, 3, "near_identity", 81), "f32")
+    psi = synth.round_to(synth.spinor(L, Nv, 4, 3, 82), prec)
+    D = dg.Dirac("wilson", L, Nv, 0.12, prec)
+    D.set_links(torch.from_numpy(V).cuda())
+    Vs = synth.round_to(V, prec)
+    x = torch.from_numpy(psi.astype(np.complex64)).cuda()
+    for fmt in (0, 1):
+        D.set_link_format(fmt)
+        for variant in (1, 6):
+            if not dg.config_supported("wilson", prec, 2, 32, variant, L):
+                continue
+            D.set_kernel_config(2, 32, variant)
+            for dag in (False, True):
+                got = D.apply(x, dagger=dag).cpu().numpy().astype(np.complex128)
+                want = oracle.apply("wilson", Vs, psi, oracle.kappa_to_m0(0.12), dagger=dag)
+                assert rel_l2(got, want) <= TOL[prec], (fmt, variant, dag)
+    D.close()
