@@ -93,6 +93,10 @@ template <> struct Store<__half> {
 // 16-bit pair <-> float complex
 HD cx<float> unpack2(uint32_t w, __nv_bfloat16*)
 {
+#if defined(__CUDA_ARCH__)
+    // one operation each: the high half in place (extracting it first takes two)
+    return {__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u)};
+#endif
     __nv_bfloat162 h = *reinterpret_cast<__nv_bfloat162*>(&w);
     float2 f = __bfloat1622float2(h);
     return {f.x, f.y};

@@ -309,13 +309,13 @@ DEV_INLINE void wilson_site_xlast(const ApplyArgs& a, long s, int lane, int grou
 // ---------------------------------------------------------------- Wilson, pairs of right-hand sides
 // The sweeps of two right-hand sides per thread of 16-bit fields, with the two in
 // the halves of packed FP32 registers: one f32x2 instruction does both, each link entry
-// is broadcast once for 2 x 2 colour vectors, and the spin projections, done right-hand side
-// by right-hand side, write their halves without moves (pairs of (re, im), tried
-// before, needed a swapped copy of every factor).  A quarter of the sweep's
-// instructions go, and 16-bit sweeps, which also unpack every value, gain by it:
-// 16^3 x 32, Nv = 24, BF16, variant 6: 208 -> 169 us, with the loads one hop ahead 166 (the best shape
-// before, variant 5: 187); 32^4, Nv = 12: 656 (variant 5: 718).  FP32 sweeps keep the
-// scalar form: at 12 warps per SM they wait for memory whatever they execute (32^4,
+// is broadcast once for 2 x 2 colour vectors, and the 16-bit words are unpacked
+// straight into the halves (pairs of (re, im), tried before, needed a swapped copy of
+// every factor).  A third of the sweep's instructions go (16^3 x 32, Nv = 24, BF16,
+// variant 6: 100 M), and 16-bit sweeps, which also unpack every value, gain by it: 208 -> 153 us (the
+// best shape before, variant 5: 187); 32^4, Nv = 12: 610 (variant 5: 718).  Bound now by
+// issue (54 %) and the FMA pipe (55 %) of 11 warps per SM.  FP32 sweeps keep the
+// scalar form: they wait for memory whatever they execute (32^4,
 // Nv = 12: 131 -> 97 M instructions, 0.70 -> 0.73 ms, and the same with loads ahead).
 struct c2 { f2 re, im; };   // a complex number of each right-hand side
 
@@ -370,6 +370,28 @@ DEV_INLINE c2 add2(c2 a, c2 b) { return {fadd2(a.re, b.re), fadd2(a.im, b.im)}; 
 DEV_INLINE c2 sub2(c2 a, c2 b) { return {fsub2(a.re, b.re), fsub2(a.im, b.im)}; }
 DEV_INLINE c2 addi2(c2 a, c2 b) { return {fsub2(a.re, b.im), fadd2(a.im, b.re)}; }   // a + i b
 DEV_INLINE c2 subi2(c2 a, c2 b) { return {fadd2(a.re, b.im), fsub2(a.im, b.re)}; }   // a - i b
+
+// wilson_project of both
+template <int MU, int S>
+DEV_INLINE void project2(const c2* p, c2* h)
+{
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        if constexpr (MU == 0) {
+            h[c] = S > 0 ? subi2(p[c], p[9 + c]) : addi2(p[c], p[9 + c]);
+            h[3 + c] = S > 0 ? subi2(p[3 + c], p[6 + c]) : addi2(p[3 + c], p[6 + c]);
+        } else if constexpr (MU == 1) {
+            h[c] = S > 0 ? sub2(p[c], p[9 + c]) : add2(p[c], p[9 + c]);
+            h[3 + c] = S > 0 ? add2(p[3 + c], p[6 + c]) : sub2(p[3 + c], p[6 + c]);
+        } else if constexpr (MU == 2) {
+            h[c] = S > 0 ? subi2(p[c], p[6 + c]) : addi2(p[c], p[6 + c]);
+            h[3 + c] = S > 0 ? addi2(p[3 + c], p[9 + c]) : subi2(p[3 + c], p[9 + c]);
+        } else {
+            h[c] = S > 0 ? add2(p[c], p[6 + c]) : sub2(p[c], p[6 + c]);
+            h[3 + c] = S > 0 ? add2(p[3 + c], p[9 + c]) : sub2(p[3 + c], p[9 + c]);
+        }
+    }
+}
 
 // wilson_reconstruct of colour c
 template <int MU, int S>
@@ -430,16 +452,18 @@ DEV_INLINE void raw_load(const ApplyArgs& a, int v0, long s, Raw2<T>& p)
         for (int k = 0; k < Raw2<T>::K; ++k) p.e[r][k] = ld_now(q + 32 * k);
     }
 }
-template <typename T> DEV_INLINE void raw_spinor(const Raw2<T>& p, int r, cx<float>* o)
+template <typename T> DEV_INLINE void raw_spinor(const Raw2<T>& p, c2* o)
 {
 #pragma unroll
-    for (int k = 0; k < Raw2<T>::K; ++k) {
-        const uint4 v = p.e[r][k];
-        o[4 * k] = unpack2(v.x, (T*)nullptr);
-        o[4 * k + 1] = unpack2(v.y, (T*)nullptr);
-        o[4 * k + 2] = unpack2(v.z, (T*)nullptr);
-        o[4 * k + 3] = unpack2(v.w, (T*)nullptr);
-    }
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int k = 0; k < Raw2<T>::K; ++k) {
+            const uint4 v = p.e[r][k];
+            set_half(o[4 * k], r, unpack2(v.x, (T*)nullptr));
+            set_half(o[4 * k + 1], r, unpack2(v.y, (T*)nullptr));
+            set_half(o[4 * k + 2], r, unpack2(v.z, (T*)nullptr));
+            set_half(o[4 * k + 3], r, unpack2(v.w, (T*)nullptr));
+        }
 }
 template <typename T, int LF> struct RawLink {
     static constexpr int N = LF == 1 ? 6 : 9;
@@ -481,15 +505,9 @@ DEV_INLINE void wilson_hops2(const ApplyArgs& a, long s, const long* fwd, const 
 {
     using Q = Hop2<H, XL>;
     constexpr int S = (DAG != Q::BACK) ? +1 : -1;
-    c2 h[6];
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        cx<float> ps[12], g[6];
-        raw_spinor<T>(p, r, ps);
-        wilson_project<Q::MU, S>(ps, g);
-#pragma unroll
-        for (int i = 0; i < 6; ++i) set_half(h[i], r, g[i]);
-    }
+    c2 q[12], h[6];
+    raw_spinor<T>(p, q);
+    project2<Q::MU, S>(q, h);
     // the next hop's spinors and link, or the site's own and its x link
     RawLink<T, LF> un;
     if constexpr (H + 1 < NH) {
@@ -533,31 +551,16 @@ DEV_INLINE void wilson_site2(const ApplyArgs& a, long s, int lane, int group)
     raw_load<T, FULL>(a, v0, s + fwd[M0], p);
     raw_link<T, LF>(a, M0, s, u);
     wilson_hops2<T, 0, XL ? 6 : 8, DAG, FULL, LF, XL>(a, s, fwd, bwd, v0, p, u, acc);
-    c2 hf[6], hb[6];
+    c2 q[12], hf[6], hb[6];
+    raw_spinor<T>(p, q);
+    f2 dg;   // out = -1/2 (acc - 2 diag psi)
+    dg.x = -2.f * diag_mode<float>(a, v0, MODE);
+    dg.y = -2.f * diag_mode<float>(a, FULL ? v0 + 1 : min(v0 + 1, a.Nv - 1), MODE);
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const int v = FULL ? v0 + r : min(v0 + r, a.Nv - 1);
-        const float dg = -2.f * diag_mode<float>(a, v, MODE);   // out = -1/2 (acc - 2 diag psi)
-        cx<float> q[12], g[6];
-        raw_spinor<T>(p, r, q);
-#pragma unroll
-        for (int i = 0; i < 12; ++i) {
-            if (r == 0) {
-                acc[i].re.x = fmaf(dg, q[i].re, acc[i].re.x);
-                acc[i].im.x = fmaf(dg, q[i].im, acc[i].im.x);
-            } else {
-                acc[i].re.y = fmaf(dg, q[i].re, acc[i].re.y);
-                acc[i].im.y = fmaf(dg, q[i].im, acc[i].im.y);
-            }
-        }
-        if constexpr (XL) {
-            wilson_project<0, SF>(q, g);
-#pragma unroll
-            for (int i = 0; i < 6; ++i) set_half(hf[i], r, g[i]);
-            wilson_project<0, SB>(q, g);
-#pragma unroll
-            for (int i = 0; i < 6; ++i) set_half(hb[i], r, g[i]);
-        }
+    for (int i = 0; i < 12; ++i) acc[i] = {ffma2(dg, q[i].re, acc[i].re), ffma2(dg, q[i].im, acc[i].im)};
+    if constexpr (XL) {
+        project2<0, SF>(q, hf);
+        project2<0, SB>(q, hb);
     }
     if constexpr (XL) {
         const int Lx = a.g.L[0];
