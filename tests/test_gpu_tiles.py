@@ -122,3 +122,26 @@ def test_wilson_pairs_16bit(dg, prec, L, Nv):
                 want = oracle.apply("wilson", Vs, psi, oracle.kappa_to_m0(0.12), dagger=dag)
                 assert rel_l2(got, want) <= TOL[prec], (fmt, variant, dag)
     D.close()
+
+
+# even-odd sweeps of pairs of right-hand sides against those of one: four inner iterations of two columns and of
+# each alone.  FP32 rounding through four iterations: 1e-7 x 1e3; the split fields add flips of 16-bit roundings
+# (2^-8 (F16: 2^-11) at a rate of 1e-7 / 2^-8, so 2e-5 rms each, a dozen of them, amplified 1e1)
+@pytest.mark.parametrize("prec,tol", [("f32", 1e-4), ("bf16", 3e-3), ("f16", 3e-3)])
+@pytest.mark.parametrize("L", [(4, 4, 2, 4), (6, 2, 4, 10)])
+def test_even_odd_pairs(dg, prec, tol, L):
+    V = torch.from_numpy(synth.round_to(synth.gauge_links(L, 3, "near_identity", 91), "f32")).cuda()
+    b = synth.spinor(L, 2, 4, 3, 92)
+    xs = []
+    for cols in ((0, 1), (0,), (1,)):
+        D = dg.Dirac("wilson", L, len(cols), 0.12, prec)
+        D.set_links(V)
+        x, _, st, _ = D.solve(torch.from_numpy(np.ascontiguousarray(b[:, :, :, :, list(cols)])).cuda(), tol=1e-10,
+                              max_outer=1, max_inner=4)
+        assert st["even_odd"] == 1
+        xs.append(x.cpu().numpy())
+        D.close()
+    for v in (0, 1):
+        want = xs[1 + v][:, :, :, :, 0]
+        assert np.linalg.norm(want) > 0
+        assert np.linalg.norm(xs[0][:, :, :, :, v] - want) <= tol * np.linalg.norm(want)
