@@ -154,14 +154,15 @@ DEV_INLINE void eo_wilson_hop2(const EoArgs& a, long hn, long lsite, int v0, c2 
 {
     c2 g[6];
     if constexpr (sizeof(TI) == 2) {
+        Raw2<TI> p;
         c2 q[12];
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-            cx<float> p[12];
-            load_spinor<TI, 12>(a.in, a.vh, v0 + r, hn, p);
+            const uint4* e = static_cast<const uint4*>(a.in) + blk_index(a.vh, Raw2<TI>::K, v0 + r, 0, hn);
 #pragma unroll
-            for (int i = 0; i < 12; ++i) set_half(q[i], r, p[i]);
+            for (int k = 0; k < Raw2<TI>::K; ++k) p.e[r][k] = ld_ro(e + 32 * k);
         }
+        raw_spinor<TI>(p, q);
         project2<MU, S>(q, g);
     } else {
 #pragma unroll

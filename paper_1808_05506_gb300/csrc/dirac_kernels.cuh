@@ -459,10 +459,10 @@ template <typename T> DEV_INLINE void raw_spinor(const Raw2<T>& p, c2* o)
 #pragma unroll
         for (int k = 0; k < Raw2<T>::K; ++k) {
             const uint4 v = p.e[r][k];
-            set_half(o[4 * k], r, unpack2(v.x, (T*)nullptr));
-            set_half(o[4 * k + 1], r, unpack2(v.y, (T*)nullptr));
-            set_half(o[4 * k + 2], r, unpack2(v.z, (T*)nullptr));
-            set_half(o[4 * k + 3], r, unpack2(v.w, (T*)nullptr));
+            set_half(o[4 * k], r, unpack2_bits(v.x, (T*)nullptr));
+            set_half(o[4 * k + 1], r, unpack2_bits(v.y, (T*)nullptr));
+            set_half(o[4 * k + 2], r, unpack2_bits(v.z, (T*)nullptr));
+            set_half(o[4 * k + 3], r, unpack2_bits(v.w, (T*)nullptr));
         }
 }
 template <typename T, int LF> struct RawLink {
@@ -479,7 +479,7 @@ DEV_INLINE void raw_link(const ApplyArgs& a, int mu, long s, RawLink<T, LF>& u)
 template <typename T, int LF> DEV_INLINE void link_of(const RawLink<T, LF>& u, cx<float>* U)
 {
 #pragma unroll
-    for (int e = 0; e < RawLink<T, LF>::N; ++e) U[e] = unpack2(u.e[e], (T*)nullptr);
+    for (int e = 0; e < RawLink<T, LF>::N; ++e) U[e] = unpack2_bits(u.e[e], (T*)nullptr);
     if constexpr (LF == 1) reconstruct_row2(U);
 }
 
