@@ -37,7 +37,7 @@
 // building those in 4- and 8-byte stores (6900 instructions and 1600 wavefronts per
 // site) bounded that kernel.  16^3 x 32, BF16, one GB300: Nv = 16: 1.85 ms
 // with tcgen05 and on CUDA cores, 1.17 ms here; Nv = 12: 1.45 ms on CUDA
-// cores, 0.95 ms; Nv = 4: 0.55 and 0.47 ms.
+// cores, 1.00 ms; Nv = 4: 0.54 and 0.51 ms.
 #include <algorithm>
 #include <mutex>
 
