@@ -551,25 +551,6 @@ DEV_INLINE void mat_dag_vec_acc2(const cx<float>* U, const cx<float>* h, cx<floa
     }
 }
 
-// v with its sign flipped where bit 31 of m is set (no arithmetic: the FP64 pipe
-// of this GPU is 62 times slower than the integer one)
-HD float flip_sign(float v, uint32_t m)
-{
-#if defined(__CUDA_ARCH__)
-    return __uint_as_float(__float_as_uint(v) ^ m);
-#else
-    return (m & 0x80000000u) ? -v : v;
-#endif
-}
-HD double flip_sign(double v, uint32_t m)
-{
-#if defined(__CUDA_ARCH__)
-    return __hiloint2double(__double2hiint(v) ^ (int)m, __double2loint(v));
-#else
-    return (m & 0x80000000u) ? -v : v;
-#endif
-}
-
 // value of v held by lane src of this warp (all 32 lanes take part)
 template <typename A> DEV_INLINE cx<A> shfl_cx(cx<A> v, int src)
 {

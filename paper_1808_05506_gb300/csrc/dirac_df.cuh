@@ -119,8 +119,6 @@ HD dfl fma(dfl a, dfl b, dfl c)
 }
 HD dfl operator*(dfl a, dfl b) { return fma(a, b, dfl()); }
 
-HD dfl flip_sign(dfl a, uint32_t m) { return dfl(dirac::flip_sign(a.hi, m), dirac::flip_sign(a.lo, m)); }
-
 // the double nearest to hi + lo (exact: the two halves fit 53 bits)
 HD double df_to_double(dfl a) { return (double)a.hi + (double)a.lo; }
 

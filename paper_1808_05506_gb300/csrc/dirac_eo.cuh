@@ -232,7 +232,7 @@ DEV_INLINE void staggered_eo_site(const EoArgs& a, long h, int group, typename S
     int par = 0;  // x_0 + ... + x_{mu-1}
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
-        const uint32_t eta = (uint32_t)par << 31;
+        const A eta = (par & 1) ? A(-1) : A(1);
         par += x[mu];
         cx<A> Uf[9], Ub[9];
         load_link<TL>(a.links, a.g.vol, mu, s, Uf);
@@ -243,7 +243,7 @@ DEV_INLINE void staggered_eo_site(const EoArgs& a, long h, int group, typename S
             cx<A> pf[3], pb[3];
             load_spinor<TI, 3>(a.in, a.vh, v0 + r, hf, pf);
             load_spinor<TI, 3>(a.in, a.vh, v0 + r, hb, pb);
-            staggered_hops(Uf, Ub, pf, pb, mu == 0 ? 0u : eta, acc[r]);
+            staggered_hops(Uf, Ub, pf, pb, eta, acc[r]);
         }
     }
     const A* cf = static_cast<const A*>(a.coef);

@@ -21,37 +21,55 @@ using namespace dirac;
 
 namespace dirac {
 
-// acc[a][b] += sum_{comp} u_comp[a] conj(w_comp[b]) for NC 3-vectors
+// t[a][b] += sum_{comp} u_comp[a] conj(w_comp[b]) for NC 3-vectors
 template <int NC, typename A>
-__device__ __forceinline__ void outer_acc(cx<A>* acc, const cx<A>* u, const cx<A>* w)
+__device__ __forceinline__ void outer_products(cx<A>* t, const cx<A>* u, const cx<A>* w)
 {
 #pragma unroll
     for (int k = 0; k < NC; ++k)
 #pragma unroll
         for (int a = 0; a < 3; ++a)
 #pragma unroll
-            for (int b = 0; b < 3; ++b) acc[3 * a + b] = cfma_conj(w[3 * k + b], u[3 * k + a], acc[3 * a + b]);
+            for (int b = 0; b < 3; ++b) t[3 * a + b] = cfma_conj(w[3 * k + b], u[3 * k + a], t[3 * a + b]);
 }
 
-// acc += t (FP32), the products having gone into t; FP64: t is acc
-template <int NC, typename A>
-__device__ __forceinline__ void outer_sum(cx<A>* acc, const cx<A>* u, const cx<A>* w, const cx<A>* u2, const cx<A>* w2)
+// acc += f (u w^+ + u2 w2^+), the two hops of a link with NC components each.  f joins
+// each sum, not the end of it, which could leave the range where the result does
+// not.  What is summed by itself first, by what rounds least: both hops, or
+// (SINGLE) each component.  FP64 takes SINGLE: a sum of both hops, or straight into
+// acc, saves a third of its operations and puts the staggered force of one right-hand side
+// 8.8e-17 instead of 4.7e-17 from the exact one.  FP32 sums both hops (16 right-hand
+// sides: Wilson 1.0e-7 instead of 1.6e-7, staggered 8.7e-8 instead of 1.1e-7), except
+// Wilson with one right-hand side, where there is no longer sum to keep short (6.6e-8
+// and 6.4e-8).
+template <int NC, bool SINGLE, typename A>
+__device__ __forceinline__ void outer_sum(cx<A>* acc, A f, const cx<A>* u, const cx<A>* w, const cx<A>* u2, const cx<A>* w2)
 {
-    if constexpr (sizeof(A) == 8) {
-        outer_acc<NC>(acc, u, w);
-        outer_acc<NC>(acc, u2, w2);
-    } else {
-        cx<A> t[9];
+    cx<A> t[9];
+    auto clear = [&]() {
 #pragma unroll
         for (int e = 0; e < 9; ++e) t[e] = cx<A>{A(0), A(0)};
-        outer_acc<NC>(t, u, w);
-        outer_acc<NC>(t, u2, w2);
+    };
+    auto join = [&]() {
 #pragma unroll
-        for (int e = 0; e < 9; ++e) acc[e] = acc[e] + t[e];
+        for (int e = 0; e < 9; ++e) acc[e] = cx<A>{fma(f, t[e].re, acc[e].re), fma(f, t[e].im, acc[e].im)};
+    };
+    if constexpr (SINGLE) {
+#pragma unroll
+        for (int k = 0; k < 2 * NC; ++k) {
+            clear();
+            outer_products<1>(t, k < NC ? u + 3 * k : u2 + 3 * (k - NC), k < NC ? w + 3 * k : w2 + 3 * (k - NC));
+            join();
+        }
+    } else {
+        clear();
+        outer_products<NC>(t, u, w);
+        outer_products<NC>(t, u2, w2);
+        join();
     }
 }
 
-template <int MU, typename A>
+template <int MU, bool SINGLE, typename A>
 __device__ __forceinline__ void wilson_force_hop(cx<A>* acc, const cx<A>* gs, const cx<A>* ps, const cx<A>* gn, const cx<A>* pn)
 {
     cx<A> h[6], k[6], h2[6], k2[6];
@@ -59,19 +77,16 @@ __device__ __forceinline__ void wilson_force_hop(cx<A>* acc, const cx<A>* gs, co
     wilson_project<MU, -1>(pn, k);
     wilson_project<MU, +1>(ps, k2);
     wilson_project<MU, +1>(gn, h2);
-    outer_sum<2>(acc, h, k, k2, h2);
+    outer_sum<2, SINGLE>(acc, A(-0.5), h, k, k2, h2);
 }
 
 // The links mu = m0 .. m0 + NM - 1 of site s.  The four links of a site share
 // psi(x) and g(x): NM links in a thread load 2 + 2 NM spinors per right-hand
 // side instead of 4 NM.  FP32 and 16-bit: bound by those loads, which come from
-// L2 (16 a site at NM = 1; 16^4, Nv = 8, FP32 Wilson: NM = 1 61 us, 2 55, 4 43).  Each hop's products are
-// summed by themselves before they join the sum over right-hand sides (a chain
-// of all of them in FP32 rounds more).  FP64: bound by FP64 arithmetic,
-// 72 multiply-adds per link, right-hand side and colour pair of spinors, so the
-// products go straight into the sums and the factor -1/2 (eta / 2) to the end
-// (staggered 404 -> 265 us).
-template <typename T, int M0, int NM>
+// L2 (16 a site at NM = 1; 16^4, Nv = 8, FP32 Wilson: NM = 1 64 us, 4 44).  FP64: bound by
+// FP64 arithmetic, 108 operations per link, right-hand side and pair of 3-vectors
+// (16^4, Nv = 8: staggered 406 us, Wilson 1052).
+template <typename T, int M0, int NM, bool SINGLE>
 __device__ __forceinline__ void wilson_force_links(const Geom& g, int Nv, const void* psi, const void* gv, long s,
                                                    const long* fwd, cx<typename Store<T>::A> (&acc)[NM][9])
 {
@@ -84,15 +99,15 @@ __device__ __forceinline__ void wilson_force_links(const Geom& g, int Nv, const 
         for (int m = 0; m < NM; ++m) {
             load_spinor<T, 12>(gv, g.vol, v, s + fwd[M0 + m], gn);
             load_spinor<T, 12>(psi, g.vol, v, s + fwd[M0 + m], pn);
-            if (M0 + m == 0) wilson_force_hop<0>(acc[m], gs, ps, gn, pn);
-            else if (M0 + m == 1) wilson_force_hop<1>(acc[m], gs, ps, gn, pn);
-            else if (M0 + m == 2) wilson_force_hop<2>(acc[m], gs, ps, gn, pn);
-            else wilson_force_hop<3>(acc[m], gs, ps, gn, pn);
+            if (M0 + m == 0) wilson_force_hop<0, SINGLE>(acc[m], gs, ps, gn, pn);
+            else if (M0 + m == 1) wilson_force_hop<1, SINGLE>(acc[m], gs, ps, gn, pn);
+            else if (M0 + m == 2) wilson_force_hop<2, SINGLE>(acc[m], gs, ps, gn, pn);
+            else wilson_force_hop<3, SINGLE>(acc[m], gs, ps, gn, pn);
         }
     }
 }
 
-template <typename T, bool STAG, int NM>
+template <typename T, bool STAG, int NM, bool SINGLE>
 __global__ void __launch_bounds__(128) k_force(Geom g, int Nv, const void* psi, const void* gv, void* F)
 {
     using A = typename Store<T>::A;
@@ -108,8 +123,8 @@ __global__ void __launch_bounds__(128) k_force(Geom g, int Nv, const void* psi, 
     for (int m = 0; m < NM; ++m)
 #pragma unroll
         for (int e = 0; e < 9; ++e) acc[m][e] = cx<A>{A(0), A(0)};
-    A f[NM];
     if constexpr (STAG) {
+        A f[NM];
         long sp[NM];
 #pragma unroll
         for (int m = 0; m < NM; ++m) {
@@ -128,21 +143,19 @@ __global__ void __launch_bounds__(128) k_force(Geom g, int Nv, const void* psi, 
             for (int m = 0; m < NM; ++m) {
                 load_spinor<T, 3>(gv, g.vol, v, sp[m], gn);
                 load_spinor<T, 3>(psi, g.vol, v, sp[m], pn);
-                outer_sum<1>(acc[m], gs, pn, ps, gn);
+                outer_sum<1, SINGLE>(acc[m], f[m], gs, pn, ps, gn);
             }
         }
     } else {
-#pragma unroll
-        for (int m = 0; m < NM; ++m) f[m] = A(-0.5);
-        if constexpr (NM == 4) wilson_force_links<T, 0, 4>(g, Nv, psi, gv, s, fwd, acc);
+        if constexpr (NM == 4) wilson_force_links<T, 0, 4, SINGLE>(g, Nv, psi, gv, s, fwd, acc);
         else if constexpr (NM == 2) {
-            if (q == 0) wilson_force_links<T, 0, 2>(g, Nv, psi, gv, s, fwd, acc);
-            else wilson_force_links<T, 2, 2>(g, Nv, psi, gv, s, fwd, acc);
+            if (q == 0) wilson_force_links<T, 0, 2, SINGLE>(g, Nv, psi, gv, s, fwd, acc);
+            else wilson_force_links<T, 2, 2, SINGLE>(g, Nv, psi, gv, s, fwd, acc);
         } else {
-            if (q == 0) wilson_force_links<T, 0, 1>(g, Nv, psi, gv, s, fwd, acc);
-            else if (q == 1) wilson_force_links<T, 1, 1>(g, Nv, psi, gv, s, fwd, acc);
-            else if (q == 2) wilson_force_links<T, 2, 1>(g, Nv, psi, gv, s, fwd, acc);
-            else wilson_force_links<T, 3, 1>(g, Nv, psi, gv, s, fwd, acc);
+            if (q == 0) wilson_force_links<T, 0, 1, SINGLE>(g, Nv, psi, gv, s, fwd, acc);
+            else if (q == 1) wilson_force_links<T, 1, 1, SINGLE>(g, Nv, psi, gv, s, fwd, acc);
+            else if (q == 2) wilson_force_links<T, 2, 1, SINGLE>(g, Nv, psi, gv, s, fwd, acc);
+            else wilson_force_links<T, 3, 1, SINGLE>(g, Nv, psi, gv, s, fwd, acc);
         }
     }
     if constexpr (sizeof(A) == 4 && NM > 1) {
@@ -151,8 +164,7 @@ __global__ void __launch_bounds__(128) k_force(Geom g, int Nv, const void* psi, 
 #pragma unroll
         for (int e = 0; e < NM * 9; e += 2) {
             const cx<A> c0 = acc[e / 9][e % 9], c1 = acc[(e + 1) / 9][(e + 1) % 9];
-            const A f0 = f[e / 9], f1 = f[(e + 1) / 9];
-            out[e / 2] = make_float4(f0 * c0.re, f0 * c0.im, f1 * c1.re, f1 * c1.im);
+            out[e / 2] = make_float4(c0.re, c0.im, c1.re, c1.im);
         }
     } else {
         using O = typename Store<A>::One;   // float2 or double2
@@ -160,18 +172,18 @@ __global__ void __launch_bounds__(128) k_force(Geom g, int Nv, const void* psi, 
 #pragma unroll
         for (int e = 0; e < NM * 9; ++e) {
             O o;
-            o.x = f[e / 9] * acc[e / 9][e % 9].re;
-            o.y = f[e / 9] * acc[e / 9][e % 9].im;
+            o.x = acc[e / 9][e % 9].re;
+            o.y = acc[e / 9][e % 9].im;
             out[e] = o;
         }
     }
 }
 
-template <typename T, bool STAG, int NM>
+template <typename T, bool STAG, int NM, bool SINGLE>
 static cudaError_t force_go(const Geom& g, int Nv, const void* psi, const void* gv, void* F, cudaStream_t st)
 {
     const long n = (4 / NM) * g.vol;
-    k_force<T, STAG, NM><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(g, Nv, psi, gv, F);
+    k_force<T, STAG, NM, SINGLE><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(g, Nv, psi, gv, F);
     return cudaGetLastError();
 }
 
@@ -180,11 +192,12 @@ template <typename T>
 static cudaError_t force_T(int op, const Geom& g, int Nv, const void* psi, const void* gv, void* F, cudaStream_t st)
 {
     if constexpr (sizeof(T) == 8) {
-        if (op == OP_STAGGERED) return force_go<T, true, 1>(g, Nv, psi, gv, F, st);
-        return force_go<T, false, 1>(g, Nv, psi, gv, F, st);
+        if (op == OP_STAGGERED) return force_go<T, true, 1, true>(g, Nv, psi, gv, F, st);
+        return force_go<T, false, 1, true>(g, Nv, psi, gv, F, st);
     } else {
-        if (op == OP_STAGGERED) return force_go<T, true, 4>(g, Nv, psi, gv, F, st);
-        return force_go<T, false, 4>(g, Nv, psi, gv, F, st);
+        if (op == OP_STAGGERED) return force_go<T, true, 4, false>(g, Nv, psi, gv, F, st);
+        if (Nv == 1) return force_go<T, false, 4, true>(g, Nv, psi, gv, F, st);
+        return force_go<T, false, 4, false>(g, Nv, psi, gv, F, st);
     }
 }
 

@@ -965,40 +965,27 @@ DEV_INLINE void wilson_site_pipe(const ApplyArgs& a, long s, int group, char* sm
 }
 
 // ---------------------------------------------------------------- staggered
-// acc += eta (Uf pf - Ub^+ pb), the sign eta in bit 31.  FP32: the two hops of a
-// direction are summed before they join the others (a chain of all 24 products
-// of a component rounds half again as much).  FP64 and double-float: eta is a
-// sign flip of the spinors and the products go straight into the sums.
+// acc += eta (Uf pf - Ub^+ pb).  The two hops of a direction
+// are summed before they join the others, in every arithmetic: a chain of all 24
+// products of a component, which saves 48 of 348 FP64 operations per site and
+// right-hand side, rounds nearly twice as much (8^4, Nv = 4, FP64: 2.7e-16
+// against 1.4e-16 of the result).
 template <typename A>
-DEV_INLINE void staggered_hops(const cx<A>* Uf, const cx<A>* Ub, cx<A>* pf, cx<A>* pb, uint32_t eta, cx<A>* acc)
+DEV_INLINE void staggered_hops(const cx<A>* Uf, const cx<A>* Ub, const cx<A>* pf, const cx<A>* pb, A eta, cx<A>* acc)
 {
-    const uint32_t m = eta & 0x80000000u;
-    if constexpr (std::is_same<A, float>::value) {
-        const float e = m ? -1.f : 1.f;
-        cx<A> w[3], wb[3];
-        mat_vec(Uf, pf, w);
-        mat_dag_vec(Ub, pb, wb);
+    cx<A> w[3], wb[3];
+    mat_vec(Uf, pf, w);
+    mat_dag_vec(Ub, pb, wb);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const cx<A> d = w[c] - wb[c];
-            acc[c].re = fma(e, d.re, acc[c].re);
-            acc[c].im = fma(e, d.im, acc[c].im);
-        }
-    } else {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            pf[c] = cx<A>{flip_sign(pf[c].re, m), flip_sign(pf[c].im, m)};
-            pb[c] = cx<A>{flip_sign(pb[c].re, m ^ 0x80000000u), flip_sign(pb[c].im, m ^ 0x80000000u)};
-        }
-        mat_vec_acc(Uf, pf, acc);
-        mat_dag_vec_acc(Ub, pb, acc);
+    for (int c = 0; c < 3; ++c) {
+        const cx<A> d = w[c] - wb[c];
+        acc[c].re = fma(eta, d.re, acc[c].re);
+        acc[c].im = fma(eta, d.im, acc[c].im);
     }
 }
 
-// MODE and LF as in wilson_site.  FP64: 288 multiply-adds and 12 operations for
-// the diagonal (348 operations with the hops summed by themselves) per site and
-// right-hand side, which is what bounds the sweep (16^4, Nv = 8: 322 -> 272 us, 0.59 T
-// operations per second).
+// MODE and LF as in wilson_site.  FP64: bound by its 348 operations per site and
+// right-hand side (16^4, Nv = 8: 324 us).
 template <typename T, int R, bool DAG, int MODE = 0, int LF = 0, bool CANON = false>
 DEV_INLINE void staggered_site(const ApplyArgs& a, long s, int group, OutTo to = OutTo())
 {
@@ -1016,7 +1003,7 @@ DEV_INLINE void staggered_site(const ApplyArgs& a, long s, int group, OutTo to =
     int par = 0;  // x_0 + ... + x_{mu-1}
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
-        const uint32_t eta = (uint32_t)par << 31;
+        const A eta = (par & 1) ? A(-1) : A(1);
         par += x[mu];
         cx<A> Uf[9], Ub[9];
         load_link_f<T, false, LF>(a.links, a.g.vol, mu, s, Uf);
@@ -1027,7 +1014,7 @@ DEV_INLINE void staggered_site(const ApplyArgs& a, long s, int group, OutTo to =
             cx<A> pf[3], pb[3];
             load_spinor<T, 3>(a.in, a.g.vol, v, s + fwd[mu], pf);
             load_spinor<T, 3>(a.in, a.g.vol, v, s + bwd[mu], pb);
-            staggered_hops(Uf, Ub, pf, pb, mu == 0 ? 0u : eta, acc[r]);
+            staggered_hops(Uf, Ub, pf, pb, eta, acc[r]);
         }
     }
     const A hf = DAG ? A(-0.5) : A(0.5);
@@ -1076,7 +1063,7 @@ DEV_INLINE void staggered_site_xlast(const ApplyArgs& a, long s, int lane, int g
     int par = x[0];  // x_0 + ... + x_{mu-1}, from mu = 1 on
 #pragma unroll
     for (int mu = 1; mu < 4; ++mu) {
-        const uint32_t eta = (uint32_t)par << 31;
+        const A eta = (par & 1) ? A(-1) : A(1);
         par += x[mu];
         cx<A> Uf[9], Ub[9];
         load_link_f<T, false, LF>(a.links, a.g.vol, mu, s, Uf);
@@ -1087,7 +1074,7 @@ DEV_INLINE void staggered_site_xlast(const ApplyArgs& a, long s, int lane, int g
             cx<A> pf[3], pb[3];
             load_spinor<T, 3>(a.in, a.g.vol, v, s + fwd[mu], pf);
             load_spinor<T, 3>(a.in, a.g.vol, v, s + bwd[mu], pb);
-            staggered_hops(Uf, Ub, pf, pb, mu == 0 ? 0u : eta, acc[r]);
+            staggered_hops(Uf, Ub, pf, pb, eta, acc[r]);
         }
     }
     cx<A> U[9];
