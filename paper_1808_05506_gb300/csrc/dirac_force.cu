@@ -187,7 +187,29 @@ static cudaError_t force_go(const Geom& g, int Nv, const void* psi, const void* 
     return cudaGetLastError();
 }
 
-// links per thread: FP64 one (144 registers of sums for four)
+// share of the block slots that a launch of vol / 128 * (4 / NM) blocks keeps busy, `per`
+// blocks to an SM (152 SMs)
+static double last_wave(long vol, int NM, int per)
+{
+    const long blocks = ((4 / NM) * vol + 127) / 128, slots = 152L * per;
+    return (double)blocks / ((blocks + slots - 1) / slots * slots);
+}
+
+// Links per thread NM.  FP64: one (144 registers of sums for four).  Else four read least
+// but leave a quarter of the threads, two blocks to an SM (Wilson): small lattices, and
+// those whose last wave is mostly empty, take fewer.  The lines lie where the
+// next lower NM, or NM = 1, the kernel of one link per thread, is as fast for every Nv
+// from 1 to 24 (us for NM = 1, 2, 4, Nv = 12): Wilson F32 10^4 20 29 19, 12^4 27 26 27,
+// 16^3 x 8 39 49 27, 16^4 103 93 62, 24^4 533 372 277; BF16 8^4 11 15 19, 12^4 23 25 29, 16^3 x 12 43 41
+// 43 (Nv = 24: 92 97 101), 24^4 309 279 253; staggered F32 8^4 9 10 15, 12^4 13 13 20, 16^4 27 23 27,
+// 24^4 197 130 131 (Nv = 3: 115 61 51).
+static int links_per_thread(int op, bool f32, long vol)
+{
+    if (op == OP_STAGGERED) return vol < 16384 ? 1 : (vol < 200000 ? 2 : 4);
+    if (last_wave(vol, 4, 2) >= (f32 ? 0.6 : 0.75)) return 4;
+    return f32 && last_wave(vol, 2, 3) >= 0.7 ? 2 : 1;
+}
+
 template <typename T>
 static cudaError_t force_T(int op, const Geom& g, int Nv, const void* psi, const void* gv, void* F, cudaStream_t st)
 {
@@ -195,8 +217,16 @@ static cudaError_t force_T(int op, const Geom& g, int Nv, const void* psi, const
         if (op == OP_STAGGERED) return force_go<T, true, 1, true>(g, Nv, psi, gv, F, st);
         return force_go<T, false, 1, true>(g, Nv, psi, gv, F, st);
     } else {
-        if (op == OP_STAGGERED) return force_go<T, true, 4, false>(g, Nv, psi, gv, F, st);
-        if (Nv == 1) return force_go<T, false, 4, true>(g, Nv, psi, gv, F, st);
+        const int nm = links_per_thread(op, sizeof(T) == 4, g.vol);
+        if (op == OP_STAGGERED) {
+            if (nm == 1) return force_go<T, true, 1, false>(g, Nv, psi, gv, F, st);
+            if (nm == 2) return force_go<T, true, 2, false>(g, Nv, psi, gv, F, st);
+            return force_go<T, true, 4, false>(g, Nv, psi, gv, F, st);
+        }
+        if (Nv == 1) return force_go<T, false, 1, true>(g, Nv, psi, gv, F, st);
+        if (nm == 1) return force_go<T, false, 1, false>(g, Nv, psi, gv, F, st);
+        if constexpr (sizeof(T) == 4)
+            if (nm == 2) return force_go<T, false, 2, false>(g, Nv, psi, gv, F, st);
         return force_go<T, false, 4, false>(g, Nv, psi, gv, F, st);
     }
 }
