@@ -778,50 +778,65 @@ bool apply_config_supported(int op, int prec, int R, int block, int variant, con
     return op == OP_WILSON && variant == V_PIPE3 && wilson_pipe_smem(prec, R, block, 3) <= 227 * 1024;
 }
 
+// share of an SM's 384 resident threads (168 registers each) that work on a right-hand side
+// when a sweep takes ng groups in blocks of `block` sites
+static double groups_fill(int block, int ng)
+{
+    const int gy = groups_per_block(block, ng), threads = block * gy;
+    return (double)ng / ((ng + gy - 1) / gy * gy) * (384 / threads * threads) / 384.0;
+}
+
 // The launch shape of a handle that was not tuned.  Wilson and staggered sweeps of
 // FP32 and 16-bit storage are bound by what they read through L2, so the shapes
 // that read least come first: x hops last by lane exchange (variant 6) where
 // the lattice allows it, else the groups of a site in one block (variant 1).
-// Right-hand sides per thread R: the largest that leaves little of the last
-// block's groups empty.  Lexicographic order, except where a t-slice and
-// its result take more than 25 MB, a good part of the L2 (then t-chunks).
-// Measured against variant 0, R dividing Nv, 128 threads (FP32, us):
-//   Wilson 16^3x32 Nv = 12 109 -> 94, 32x16^3 Nv = 8 76 -> 65, 32^4 Nv = 12
-//   1010 -> 777, 24^4 Nv = 12 297 -> 253, 20x18x16x24 Nv = 5 64 -> 62;
-//   staggered 16^3x32 Nv = 12 51 -> 39, 32^4 Nv = 4 130 -> 101, Nv = 3 148 -> 108,
-//   24^4 Nv = 12 114 -> 95, 16x18x20x32 Nv = 24 122 -> 101.
+// Right-hand sides per thread R and sites per block: those that leave little of the
+// blocks and of the SM empty; where variant 1 leaves more than 15 %, and for F16 Wilson
+// with an odd Nv (a pair would compute one for nothing, and variant 1 gains
+// nothing there by itself), variant 0.
+// Lexicographic order, except where a t-slice and its result take more than 25 MB, a
+// good part of the L2 (then t-chunks).
+// Measured against variant 0, R dividing Nv, 128 threads, on 15 lattices of 4^3 to 32^3 x 16 and
+// Nv = 1..24 (geometric mean of the ratio of times, and the largest above 20 us):
+//   Wilson F32 0.90, 1.06, BF16 0.84, 1.00, F16 0.94, 1.00;
+//   staggered F32 0.85, 1.00, BF16 0.93, 1.01, F16 0.92, 1.02;
+// with weights for all of them that FP32 was measured for, and 64 sites per block in variant 1:
+// F16 Wilson 24^4 Nv = 7 1.37, staggered Nv = 16 1.2.
 // FP64 and Brillouin sweeps are bound by arithmetic: variant 0.
 LaunchCfg default_config(int op, int prec, int Nv, const Geom* g)
 {
-    if (op == OP_BRILLOUIN || prec == P_F64 || !g) {
-        if (op == OP_STAGGERED) {
-            int R = (Nv % 6 == 0) ? 6 : (Nv % 4 == 0 ? 4 : (Nv % 2 == 0 ? 2 : 1));
-            if (prec == P_F64 && R > 4) R = 4;
-            return LaunchCfg{R, 128, V_DIRECT};
-        }
-        return LaunchCfg{(Nv % 2 == 0) ? 2 : 1, 128, V_DIRECT};
+    LaunchCfg direct{(Nv % 2 == 0) ? 2 : 1, 128, V_DIRECT};
+    if (op == OP_STAGGERED) {
+        direct.R = (Nv % 6 == 0) ? 6 : (Nv % 4 == 0 ? 4 : (Nv % 2 == 0 ? 2 : 1));
+        if (prec == P_F64 && direct.R > 4) direct.R = 4;
     }
+    if (op == OP_BRILLOUIN || prec == P_F64 || !g) return direct;
     const bool xlast = 32 % g->L[0] == 0 && g->stride[3] % 32 == 0;
-    const int block = xlast ? 32 : 64;
-    const double slice = (double)g->stride[3] * Nv * nsc_of(op) * cbytes(prec);
-    const int order = slice > 25e6 ? (g->L[3] < 8 ? g->L[3] : 8) : 0;
-    int R = 1;
+    if (op == OP_WILSON && prec == P_F16 && Nv % 2 && !xlast) return direct;
+    int R = 1, block = 32;
     if (op == OP_WILSON) {
         R = (Nv % 2 == 0 || Nv >= 5) ? 2 : 1;
+        const int ng = (Nv + R - 1) / R;
+        if (ng > 3 && groups_fill(64, ng) >= groups_fill(32, ng)) block = 64;
     } else {
         // right-hand sides the blocks compute, times what a thread of few costs more
         double best = 0.0;
         const int Rs[] = {6, 4, 2, 1};
         const double f[] = {xlast ? 1.05 : 1.0, 1.0, 1.1, 1.5};
-        for (int i = 0; i < 4; ++i) {
-            const int ng = (Nv + Rs[i] - 1) / Rs[i], gy = groups_per_block(block, ng);
-            const double cost = (double)((ng + gy - 1) / gy * gy) * Rs[i] * f[i];
-            if (best == 0.0 || cost < best) {
-                best = cost;
-                R = Rs[i];
+        for (int b = xlast ? 32 : 64; b >= 32; b -= 32)
+            for (int i = 0; i < 4; ++i) {
+                const int ng = (Nv + Rs[i] - 1) / Rs[i], gy = groups_per_block(b, ng);
+                const double cost = (double)((ng + gy - 1) / gy * gy) * Rs[i] * f[i];
+                if (best == 0.0 || cost < best) {
+                    best = cost;
+                    R = Rs[i];
+                    block = b;
+                }
             }
-        }
     }
+    if (!xlast && groups_fill(block, (Nv + R - 1) / R) < 0.85) return direct;
+    const double slice = (double)g->stride[3] * Nv * nsc_of(op) * cbytes(prec);
+    const int order = slice > 25e6 ? (g->L[3] < 8 ? g->L[3] : 8) : 0;
     return LaunchCfg{R, block, xlast ? V_XLAST : V_GROUPS, order};
 }
 
