@@ -338,6 +338,32 @@ static dirac_status eo_split_sweep(dirac_handle* h, SolverWS* w, int kind, int p
                    "solve: fused norm");
 }
 
+// Launch shape of the split Brillouin sweeps of a handle that is configured for
+// the tensor cores, which has none for these CUDA-core sweeps: right-hand sides per
+// thread R by the waves of 128-thread blocks (3, 2, 2 blocks fit an SM for R = 1, 2, 3), a wave
+// costing 1, 1.1, 1.3 and the last one 0.7 of that and the rest by its fill; up to four
+// right-hand sides in groups of one, if R = 1 wins, in blocks of 32 sites.  On 8
+// lattices of 4^3 x 8 to 16^4, W = 1..24, a solve takes at most 8 % longer than with the best of
+// 17 shapes (8^4, W = 3: 6.7 ms in groups of one, 8.1 R = 2, 9.5 R = 3; W = 16: 11.7 R = 2, 14.3 R = 3;
+// 12^3 x 24, W = 12: 95.3 ms R = 3, 101 R = 2).
+static LaunchCfg split_shape(long vol, int W)
+{
+    const int resident[] = {3, 2, 2};
+    const double cost[] = {1.0, 1.1, 1.3};
+    int R = 1;
+    double best = 0.0;
+    for (int r = 1; r <= 3 && r <= W; ++r) {
+        const long blocks = (vol + 127) / 128 * ((W + r - 1) / r), slots = 152L * resident[r - 1];
+        const double rest = (double)(blocks % slots) / slots;
+        const double waves = std::max(1.0, (double)(blocks / slots) + (rest > 0.0 ? 0.7 + 0.3 * rest : 0.0));
+        if (r == 1 || waves * cost[r - 1] < best) {
+            best = waves * cost[r - 1];
+            R = r;
+        }
+    }
+    return R == 1 && W <= 4 ? LaunchCfg{1, 32, V_GROUPS} : LaunchCfg{R, 128, V_DIRECT};
+}
+
 // out = D in (or D^+ in) on the whole lattice (the inner operator without the
 // even-odd split)
 static dirac_status apply_inner_whole(dirac_handle* h, SolverWS* w, bool dag, void* out, const void* in,
@@ -355,11 +381,7 @@ static dirac_status apply_inner_whole(dirac_handle* h, SolverWS* w, bool dag, vo
     const void* L32 = nullptr;
     dirac_status st;
     if ((st = h->ensure_links32(&L32))) return st;
-    // a handle tuned to the tensor cores has no shape for these CUDA-core sweeps:
-    // three right-hand sides per thread, or two where the last group would be
-    // mostly empty (12^3 x 24, Nv = 12: 0.49 ms at R = 3, 0.67 ms at R = 1)
-    if (c0.variant == V_TC)
-        c0 = LaunchCfg{(w->W + 2) / 3 * 3 * 8 <= w->W * 9 ? 3 : 2, 128, V_DIRECT, std::min(8, h->g.L[3])};
+    if (c0.variant == V_TC) c0 = split_shape(h->g.vol, w->W);
     ApplyArgs a = h->args(out, in, w->W, h->diag);
     a.links = L32;
     a.diag_v = diag_v;
