@@ -436,7 +436,9 @@ cudaError_t tc_go_nt(bool dag, const ApplyArgs& a, int nvb, cudaStream_t st)
     if (G.nitems >= (1L << 31)) return cudaErrorInvalidValue;   // item numbers are 31 bits
     const int threads = 32 * G.bx * G.by;
     auto kern = k_brillouin_tc<T, NT>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the attribute is the kernel's, shared by all handles and host threads: always the same
+    // value, so that no thread takes back what another is about to launch with
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room);
     if (e != cudaSuccess) return e;
     int dev = 0, nsm = 0, per = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
