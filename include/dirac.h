@@ -119,8 +119,9 @@ DIRAC_API dirac_status dirac_set_stream(dirac_handle* h, void* stream);
  *   on_device  1: V is a device pointer; 0: a host pointer (copied)
  * Converts to the internal layout in the storage precision and, for
  * Brillouin, builds the 40 stored off-axis links W_dir of Tab. tab:off-axis
- * (the average over the k! hop orderings, computed in FP64 (FP64 handles) or
- * double-float arithmetic by the recursion
+ * (the average over the k! hop orderings, computed in FP64 (FP64 handles, and
+ * links whose averages leave FP32's range on the way) or double-float arithmetic
+ * by the recursion
  * W_dir(x) = (1/k) sum_{hops a} V_a(x) W_{dir-a}(x+a), then rounded).
  * Synchronous: returns after the links are in place.  The caller keeps
  * ownership of V. */
@@ -178,8 +179,8 @@ DIRAC_API dirac_status dirac_apply_dagger(dirac_handle* h, void* out, const void
  *                                -1/2 sum_v,s psi_v(x)_s [(1+gamma_mu) g_v(x+mu)]_s^+
  * Brillouin (Sec. 5, Tab. tab:off-axis): through the transporters W, which
  *   are rebuilt from V here (not kept from the forward pass; FP64 handles in
- *   FP64, the others in double-float arithmetic, 48-bit significands in
- *   FP32's exponent range, rounded to FP32 once at the end):
+ *   FP64, the others in double-float, 48-bit significands, rounded to FP32 once
+ *   at the end, and once more in FP64 where an entry would leave FP32's range on the way):
  *   G_dir(y) = sum_v,s g_v(y)_s (M_dir psi_v(y+dir))_s^+ is passed down the
  *   recursion W_dir(x) = (1/k) sum_a H_a(x) W_{dir-a}(x+a) to the links.
  *   Takes scratch of 121 * 9 complex doubles per site (17.4 KB per site) during

@@ -265,6 +265,8 @@ dirac_handle::~dirac_handle()
 {
     void* e = dev_err;
     release(e);
+    e = range_flag;
+    release(e);
     release(links);
     release(links64);
     release(W64);
@@ -356,17 +358,25 @@ dirac_status dirac_set_links(dirac_handle* h, const void* V, dirac_prec V_prec, 
             if ((st = h->build_W64())) return st;
             st = h->cuda(launch_convert_links(h->prec, h->g, 40, h->W64, h->links, h->stream), "W conversion");
         } else {
-            // W rounded to FP32 or less: built in double-float (the solver builds FP64 W on demand)
+            // W rounded to FP32 or less: built in double-float (the solver builds FP64 W on demand),
+            // again in FP64 if an entry left the range
             void* W = nullptr;
             if ((st = h->scratch((size_t)h->g.vol * 40 * 9 * 16, &W))) return st;
-            st = h->cuda(launch_build_W(h->g, h->links64, W, true, h->stream), "W build");
-            if (!st) st = h->cuda(launch_convert_links_df(h->prec, h->g, 40, W, h->links, h->stream), "W conversion");
             // the FP32 copy of the split inner solve is refreshed in place (a
             // captured solver graph holds its address)
-            if (!st && h->links32 && h->links32 != h->links) {
-                st = h->cuda(launch_convert_links_df(P_F32, h->g, 40, W, h->links32, h->stream), "FP32 W (blocked)");
-                if (!st) st = h->cuda(launch_brillouin_w80(P_F32, h->g, h->links32, h->links32, h->stream), "FP32 W, 80 directions");
+            void* L32 = h->links32 != h->links ? h->links32 : nullptr;
+            bool again = false;
+            st = h->clear_range_flag();
+            if (!st) st = h->cuda(launch_build_W(h->g, h->links64, W, true, h->stream), "W build");
+            if (!st) st = h->cuda(launch_convert_W_df(h->prec, h->g, W, h->links, h->range_flag, h->stream), "W conversion");
+            if (!st && L32) st = h->cuda(launch_convert_W_df(P_F32, h->g, W, L32, h->range_flag, h->stream), "FP32 W (blocked)");
+            if (!st) st = h->read_range_flag(&again);
+            if (!st && again) {
+                st = h->cuda(launch_build_W(h->g, h->links64, W, false, h->stream), "W build");
+                if (!st) st = h->cuda(launch_convert_links(h->prec, h->g, 40, W, h->links, h->stream), "W conversion");
+                if (!st && L32) st = h->cuda(launch_convert_links(P_F32, h->g, 40, W, L32, h->stream), "FP32 W (blocked)");
             }
+            if (!st && L32) st = h->cuda(launch_brillouin_w80(P_F32, h->g, L32, L32, h->stream), "FP32 W, 80 directions");
             h->scratch_done();
         }
         if (st) return st;
@@ -539,6 +549,24 @@ void dirac_handle::scratch_done()
         release(scr);
         scr_bytes = 0;
     }
+}
+
+dirac_status dirac_handle::clear_range_flag()
+{
+    dirac_status st;
+    void* p = range_flag;
+    if (!p && (st = alloc(&p, sizeof(int), "range flag"))) return st;
+    range_flag = static_cast<int*>(p);
+    return cuda(cudaMemsetAsync(range_flag, 0, sizeof(int), stream), "range flag");
+}
+
+dirac_status dirac_handle::read_range_flag(bool* left)
+{
+    int v = 0;
+    dirac_status st = cuda(cudaMemcpyAsync(&v, range_flag, sizeof(int), cudaMemcpyDeviceToHost, stream), "range flag");
+    if (!st) st = cuda(cudaStreamSynchronize(stream), "range flag");
+    *left = v != 0;
+    return st;
 }
 
 void dirac_handle::release_after_sync(void*& p)

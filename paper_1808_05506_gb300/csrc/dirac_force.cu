@@ -256,9 +256,21 @@ static dirac_status force_internal(dirac_handle* h, void* F, const void* pi, con
     void* scr = nullptr;
     dirac_status st;
     if ((st = h->scratch(121 * plane, &scr))) return st;
-    st = h->cuda(launch_force_brillouin(h->prec, h->g, h->Nv, pi, gi, h->links64, scr,
-                                        static_cast<char*>(scr) + 40 * plane, F, h->stream),
-                 "Brillouin force kernels");
+    auto run = [&](bool f64) {
+        return h->cuda(launch_force_brillouin(h->prec, f64, h->g, h->Nv, pi, gi, h->links64, scr,
+                                              static_cast<char*>(scr) + 40 * plane, F, h->range_flag, h->stream),
+                       "Brillouin force kernels");
+    };
+    if (h->prec == P_F64) {
+        st = run(true);
+    } else {
+        // in double-float; again in FP64 if a result left the range
+        bool again = false;
+        st = h->clear_range_flag();
+        if (!st) st = run(false);
+        if (!st) st = h->read_range_flag(&again);
+        if (!st && again) st = run(true);
+    }
     h->scratch_done();
     return st;
 }

@@ -1,7 +1,7 @@
 // Link gradient of L = Re <g, D_B psi> for the Brillouin operator (Sec. 5,
 // Eqs. def_bril, def_der, def_lap at c_SW = 0), PyTorch's convention
 // F = dL/dRe V + i dL/dIm V.  The off-axis transporters W_dir are not kept
-// between the forward and the backward pass: they are rebuilt here in FP64
+// between the forward and the backward pass: they are rebuilt here
 // from V by the recursion of Tab. tab:off-axis (every ordering of the k hops,
 // weight 1/k!, split by the first hop):
 //   W_dir(x) = (1/k) sum_{hops a of dir} H_a(x) W_{dir-a}(x+a),
@@ -16,7 +16,8 @@
 //             + sum_{dir with -mu} (1/k) W_{dir+mu}(y) G_dir(y+mu)^+
 //      (W_0 = 1: the one-hop directions).
 // Arithmetic: FP64 for FP64 handles; for the others, whose psi and g are exact
-// in FP32 and whose F is rounded to FP32, double-float (dirac_transport.cuh).
+// in FP32 and whose F is rounded to FP32, double-float (dirac_transport.cuh), and
+// FP64 after all if an entry of F leaves the range on the way.
 // All steps are bound by arithmetic (step 1: 36 complex multiply-adds per
 // direction and right-hand side, 144 FP64 operations, at a sixtieth of the
 // FP32 rate); 12^3 x 16, 8 right-hand sides, FP32 storage, one GB300:
@@ -64,8 +65,9 @@ struct Sum1 {
     __device__ __forceinline__ double get() const { return v; }
 };
 
+// one: the power of two h is kept times (kappa has it)
 template <typename A, typename S>
-__device__ __forceinline__ void h_spin(int s, const int (&d)[4], A kappa, const cx<A>* g, S (&re)[3], S (&im)[3])
+__device__ __forceinline__ void h_spin(int s, const int (&d)[4], A kappa, A one, const cx<A>* g, S (&re)[3], S (&im)[3])
 {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -75,7 +77,7 @@ __device__ __forceinline__ void h_spin(int s, const int (&d)[4], A kappa, const 
     const cx<A>* gx = g + 3 * (3 - s);
     const cx<A>* gz = g + 3 * (s ^ 2);
     if (d[0]) {   // uniform over the warp: all its threads work on one direction
-        const A f = (s < 2) ? A(d[0]) : A(-d[0]);   // -i f g
+        const A f = (s < 2) == (d[0] > 0) ? one : -one;   // -i f g
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             re[c].add(f * gx[c].im);
@@ -83,7 +85,7 @@ __device__ __forceinline__ void h_spin(int s, const int (&d)[4], A kappa, const 
         }
     }
     if (d[1]) {
-        const A f = (s == 0 || s == 3) ? A(-d[1]) : A(d[1]);
+        const A f = (s == 0 || s == 3) == (d[1] < 0) ? one : -one;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             re[c].add(f * gx[c].re);
@@ -91,7 +93,7 @@ __device__ __forceinline__ void h_spin(int s, const int (&d)[4], A kappa, const 
         }
     }
     if (d[2]) {
-        const A f = (s == 0 || s == 3) ? A(d[2]) : A(-d[2]);   // -i f g
+        const A f = (s == 0 || s == 3) == (d[2] > 0) ? one : -one;   // -i f g
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             re[c].add(f * gz[c].im);
@@ -99,7 +101,7 @@ __device__ __forceinline__ void h_spin(int s, const int (&d)[4], A kappa, const 
         }
     }
     if (d[3]) {
-        const A f = A(d[3]);
+        const A f = d[3] > 0 ? one : -one;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             re[c].add(f * gz[c].re);
@@ -108,12 +110,25 @@ __device__ __forceinline__ void h_spin(int s, const int (&d)[4], A kappa, const 
     }
 }
 
-// step 1: one thread per (site, direction j = 0..79)
-template <typename T>
+// the spinor in the arithmetic A
+template <typename T, typename A>
+__device__ __forceinline__ void load_as(const void* base, size_t vol, int v, long s, cx<A>* p)
+{
+    if constexpr (std::is_same<A, typename Store<T>::A>::value) {
+        load_spinor<T, 12>(base, vol, v, s, p);
+    } else {
+        cx<typename Store<T>::A> q[12];
+        load_spinor<T, 12>(base, vol, v, s, q);
+#pragma unroll
+        for (int i = 0; i < 12; ++i) p[i] = cx<A>{(A)q[i].re, (A)q[i].im};
+    }
+}
+
+// step 1: one thread per (site, direction j = 0..79); F64: in FP64
+template <typename T, bool F64>
 __global__ void __launch_bounds__(128) k_bri_gradW(Geom g, int Nv, const void* psi, const void* gv, void* G81)
 {
-    using A = typename Store<T>::A;                                                // of psi and g
-    constexpr bool F64 = sizeof(A) == 8;
+    using A = typename std::conditional<F64, double, float>::type;                 // of psi and g
     using B = typename std::conditional<F64, double, dfl>::type;                   // of G
     using S = typename std::conditional<F64, Sum1, Sum2>::type;
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;   // (site, j), site fastest
@@ -133,18 +148,20 @@ __global__ void __launch_bounds__(128) k_bri_gradW(Geom g, int Nv, const void* p
         nb += d[mu] > 0 ? fwd[mu] : (d[mu] < 0 ? bwd[mu] : 0);
         k += d[mu] != 0;
     }
-    const A kappa = A(-27.0 / 64.0) * A(1 << (k - 1));
+    // G of k hops is kept times 2^(f_exp - (k - 1) v_exp)
+    const A one = F64 ? A(1) : A(pow2f(f_exp<B>() - (k - 1) * v_exp<B>()));
+    const A kappa = A(-27.0 / 64.0) * A(1 << (k - 1)) * one;
     cx<B> acc[9];
 #pragma unroll
     for (int e = 0; e < 9; ++e) acc[e] = cx<B>{B(0), B(0)};
     for (int v = 0; v < Nv; ++v) {
         cx<A> ps[12], gs[12];
-        load_spinor<T, 12>(psi, g.vol, v, nb, ps);
-        load_spinor<T, 12>(gv, g.vol, v, y, gs);
+        load_as<T>(psi, g.vol, v, nb, ps);
+        load_as<T>(gv, g.vol, v, y, gs);
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
             S hr[3], hi[3];
-            h_spin<A, S>(s, d, kappa, gs, hr, hi);
+            h_spin<A, S>(s, d, kappa, one, gs, hr, hi);
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 const cx<B> h{hr[a].get(), hi[a].get()};
@@ -206,12 +223,12 @@ struct DirsOfMu {
     short code[4][54];
 };
 
-__device__ __forceinline__ float as_out(dfl a) { return a.hi; }
-__device__ __forceinline__ double as_out(double a) { return a; }
+__device__ __forceinline__ float as_out(dfl a, int* bad) { return scaled_out(a, f_exp<dfl>(), bad); }
+__device__ __forceinline__ double as_out(double a, int*) { return a; }
 
 // step 3: one thread per (site, mu); F canonical [site][mu][a][b] in the type O
 template <typename A, typename O>
-__global__ void __launch_bounds__(128) k_bri_dV(Geom g, const __grid_constant__ DirsOfMu D, const __grid_constant__ DirPlanes P, const void* G81, const void* W, O* F)
+__global__ void __launch_bounds__(128) k_bri_dV(Geom g, const __grid_constant__ DirsOfMu D, const __grid_constant__ DirPlanes P, const void* G81, const void* W, O* F, int* bad)
 {
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;   // (site, mu), site fastest
     if (i >= 4 * g.vol) return;
@@ -272,22 +289,22 @@ __global__ void __launch_bounds__(128) k_bri_dV(Geom g, const __grid_constant__ 
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
         O o;
-        o.x = as_out(F9[e].re);
-        o.y = as_out(F9[e].im);
+        o.x = as_out(F9[e].re, bad);
+        o.y = as_out(F9[e].im, bad);
         out[e] = o;
     }
 }
 
-template <typename T>
+template <typename T, bool F64>
 cudaError_t gradW_T(const Geom& g, int Nv, const void* psi, const void* gv, void* G81, cudaStream_t st)
 {
     const long n = 80 * g.vol;
-    k_bri_gradW<T><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(g, Nv, psi, gv, G81);
+    k_bri_gradW<T, F64><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(g, Nv, psi, gv, G81);
     return cudaGetLastError();
 }
 
 template <typename A, typename O>
-cudaError_t chain_T(const Geom& g, const void* W, void* G, void* F, cudaStream_t st)
+cudaError_t chain_T(const Geom& g, const void* W, void* G, void* F, int* bad, cudaStream_t st)
 {
     const DirPlanes P = dir_planes();
     for (int k = 4; k >= 2; --k) {
@@ -309,26 +326,30 @@ cudaError_t chain_T(const Geom& g, const void* W, void* G, void* F, cudaStream_t
         }
     }
     const unsigned nb = (unsigned)((4 * g.vol + 127) / 128);
-    k_bri_dV<A, O><<<nb, 128, 0, st>>>(g, D, P, G, W, static_cast<O*>(F));
+    k_bri_dV<A, O><<<nb, 128, 0, st>>>(g, D, P, G, W, static_cast<O*>(F), bad);
     return cudaGetLastError();
 }
 
 }   // namespace
 
-cudaError_t launch_force_brillouin(int prec, const Geom& g, int Nv, const void* psi, const void* gv,
-                                   const void* V64, void* W, void* G, void* F, cudaStream_t st)
+cudaError_t launch_force_brillouin(int prec, bool f64, const Geom& g, int Nv, const void* psi, const void* gv,
+                                   const void* V64, void* W, void* G, void* F, int* bad, cudaStream_t st)
 {
-    cudaError_t e = launch_build_W(g, V64, W, prec != P_F64, st);
+    f64 = f64 || prec == P_F64;
+    cudaError_t e = launch_build_W(g, V64, W, !f64, st);
     if (e != cudaSuccess) return e;
     switch (prec) {
-    case P_F64: e = gradW_T<double>(g, Nv, psi, gv, G, st); break;
-    case P_F32: e = gradW_T<float>(g, Nv, psi, gv, G, st); break;
-    case P_BF16: e = gradW_T<__nv_bfloat16>(g, Nv, psi, gv, G, st); break;
-    case P_F16: e = gradW_T<__half>(g, Nv, psi, gv, G, st); break;
+    case P_F64: e = gradW_T<double, true>(g, Nv, psi, gv, G, st); break;
+    case P_F32: e = f64 ? gradW_T<float, true>(g, Nv, psi, gv, G, st) : gradW_T<float, false>(g, Nv, psi, gv, G, st); break;
+    case P_BF16:
+        e = f64 ? gradW_T<__nv_bfloat16, true>(g, Nv, psi, gv, G, st) : gradW_T<__nv_bfloat16, false>(g, Nv, psi, gv, G, st);
+        break;
+    case P_F16: e = f64 ? gradW_T<__half, true>(g, Nv, psi, gv, G, st) : gradW_T<__half, false>(g, Nv, psi, gv, G, st); break;
     default: return cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return e;
-    return prec == P_F64 ? chain_T<double, double2>(g, W, G, F, st) : chain_T<dfl, float2>(g, W, G, F, st);
+    if (prec == P_F64) return chain_T<double, double2>(g, W, G, F, bad, st);
+    return f64 ? chain_T<double, float2>(g, W, G, F, bad, st) : chain_T<dfl, float2>(g, W, G, F, bad, st);
 }
 
 }  // namespace dirac

@@ -47,6 +47,7 @@ struct dirac_handle {
     static constexpr size_t SCRATCH_KEEP = (size_t)1 << 30;
     void* scr = nullptr;      // scratch of the W build and the Brillouin link gradient
     size_t scr_bytes = 0;
+    int* range_flag = nullptr;   // device word: a double-float chain left FP32's range (dirac_transport.cuh)
 
     // solver workspace (dirac_solve.cu)
     void* sw = nullptr;
@@ -72,6 +73,8 @@ struct dirac_handle {
     dirac_status build_W64();
     dirac_status scratch(size_t bytes, void** out);
     void scratch_done();
+    dirac_status clear_range_flag();
+    dirac_status read_range_flag(bool* left);   // waits for the stream
     dirac_status ensure_links64b(const void** out);
     dirac_status ensure_links_df(const void** out);
     dirac_status ensure_links32(const void** out);

@@ -146,9 +146,10 @@ cudaError_t launch_links_load(const Geom& g, const void* canon, bool canon_f64, 
 cudaError_t launch_convert_links(int prec, const Geom& g, int nmat, const void* src64, void* dst,
                                  cudaStream_t st);
 // Brillouin link gradient: W (40 planes) and G (81 planes) are scratch fields of 9 * vol
-// 16-byte elements per plane
-cudaError_t launch_force_brillouin(int prec, const Geom& g, int Nv, const void* psi, const void* gv,
-                                   const void* V64, void* W, void* G, void* F, cudaStream_t st);
+// 16-byte elements per plane.  f64 (always for FP64 fields): in FP64, else in
+// double-float, which sets *bad if an entry of F is not finite
+cudaError_t launch_force_brillouin(int prec, bool f64, const Geom& g, int Nv, const void* psi, const void* gv,
+                                   const void* V64, void* W, void* G, void* F, int* bad, cudaStream_t st);
 // link gradient of Re <g, D psi> (staggered, Wilson); F canonical link layout
 cudaError_t launch_force(int op, int prec, const Geom& g, int Nv, const void* psi, const void* gv, void* F,
                          cudaStream_t st);

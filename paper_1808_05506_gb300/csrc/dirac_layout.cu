@@ -257,28 +257,43 @@ cudaError_t launch_convert_links(int prec, const Geom& g, int nmat, const void* 
     return cudaGetLastError();
 }
 
-// double-float links [m][e][site] -> storage precision (FP32 or 16 bits): the
-// high half is the value rounded to FP32
+// hops of the 40 stored directions
+struct PlaneHops {
+    signed char k[40];
+};
+
+// double-float W [plane][e][site] -> storage precision (FP32 or 16 bits), rounded to FP32 first
 template <typename T>
-__global__ void k_convert_links_df(long vol, long n, const float4* __restrict__ src, void* dst)
+__global__ void k_convert_W_df(long vol, long n, const __grid_constant__ PlaneHops H, const float4* __restrict__ src, void* dst, int* bad)
 {
-    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;   // (m, e, site), site fastest
+    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;   // (plane, e, site), site fastest
     if (i >= n) return;
     const long s = i % vol;
     const long me = i / vol;
     const float4 v = src[i];
-    st_one<T>(dst, blk_index((size_t)vol, 9, (int)(me / 9), (int)(me % 9), s), cx<float>{v.x, v.z});
+    const int e = DF_V * H.k[me / 9];
+    const cx<float> c{scaled_out(dfl(v.x, v.y), e, bad), scaled_out(dfl(v.z, v.w), e, bad)};
+    st_one<T>(dst, blk_index((size_t)vol, 9, (int)(me / 9), (int)(me % 9), s), c);
 }
 
-cudaError_t launch_convert_links_df(int prec, const Geom& g, int nmat, const void* src, void* dst, cudaStream_t st)
+cudaError_t launch_convert_W_df(int prec, const Geom& g, const void* W, void* dst, int* bad, cudaStream_t st)
 {
-    const long n = g.vol * 9L * nmat;
+    BriDir dirs[80];
+    int reps[40];
+    brillouin_tables(dirs, reps);
+    PlaneHops H;
+    for (int r = 0; r < 40; ++r) {
+        int d[4];
+        dir_of(reps[r], d);
+        H.k[r] = (signed char)((d[0] != 0) + (d[1] != 0) + (d[2] != 0) + (d[3] != 0));
+    }
+    const long n = g.vol * 360L;
     const unsigned nb = (unsigned)((n + 255) / 256);
-    const float4* s = (const float4*)src;
+    const float4* s = (const float4*)W;
     switch (prec) {
-    case P_F32: k_convert_links_df<float><<<nb, 256, 0, st>>>(g.vol, n, s, dst); break;
-    case P_BF16: k_convert_links_df<__nv_bfloat16><<<nb, 256, 0, st>>>(g.vol, n, s, dst); break;
-    case P_F16: k_convert_links_df<__half><<<nb, 256, 0, st>>>(g.vol, n, s, dst); break;
+    case P_F32: k_convert_W_df<float><<<nb, 256, 0, st>>>(g.vol, n, H, s, dst, bad); break;
+    case P_BF16: k_convert_W_df<__nv_bfloat16><<<nb, 256, 0, st>>>(g.vol, n, H, s, dst, bad); break;
+    case P_F16: k_convert_W_df<__half><<<nb, 256, 0, st>>>(g.vol, n, H, s, dst, bad); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -302,7 +317,8 @@ __global__ void k_w_level1(Geom g, const __grid_constant__ DirPlanes P, const do
     const int me = (int)(i / g.vol), mu = me / 9, e = me % 9;
     int d[4] = {mu == 0, mu == 1, mu == 2, mu == 3};
     const double2 v = V64[i];
-    st_el(W, ((size_t)P.p[code_of(d)] * 9 + e) * g.vol + s, cx<A>{A(v.x), A(v.y)});
+    const double sc = (double)(1 << v_exp<A>());
+    st_el(W, ((size_t)P.p[code_of(d)] * 9 + e) * g.vol + s, cx<A>{A(sc * v.x), A(sc * v.y)});
 }
 
 template <typename A>

@@ -12,6 +12,14 @@
 // rate on this GPU and these kernels are bound by arithmetic, so for results
 // that are rounded to FP32 or less at their end double-float is the cheaper
 // arithmetic whose error (1e-14) stays far below that rounding.
+//
+// Double-float has FP32's exponent range, the result's own, but the sums on the
+// way can leave it where the result does not.  So the chain is kept times powers
+// of two, V times 2^DF_V, W of k hops times 2^(k DF_V) and the gradient times
+// 2^DF_F, which puts what its products lose below FP32's smallest number (2^-149)
+// at 2^-165 and less of the result; and a result that is not finite at the end
+// is computed again in FP64 (a word in device memory, which the host reads
+// where it waits for the stream anyway).
 #pragma once
 
 #include "dirac_df.cuh"
@@ -105,6 +113,13 @@ __device__ __forceinline__ void load_mat(const void* base, size_t vol, int plane
         }
 }
 
+// powers of two the chain is kept times (1 in FP64)
+constexpr int DF_V = 8, DF_F = 48;
+template <typename A> __device__ constexpr int v_exp() { return std::is_same<A, dfl>::value ? DF_V : 0; }
+template <typename A> __device__ constexpr int f_exp() { return std::is_same<A, dfl>::value ? DF_F : 0; }
+// 2^e, |e| <= 126
+__device__ __forceinline__ float pow2f(int e) { return __uint_as_float((uint32_t)(127 + e) << 23); }
+
 // acc += x y.  Double-float sums over many terms keep (hi, lo) unnormalised:
 // hi follows by exact two-sums, lo collects the rounding errors; settle()
 // renormalises once at the end.
@@ -153,6 +168,19 @@ __device__ __forceinline__ dfl plus(dfl a, dfl b)
     const float s = df_add(a.hi, b.hi);
     return in_range(s) ? a + b : dfl(s, 0.f);
 }
+// a 2^-e rounded to FP32 (e >= 0; below its normal range from both halves, in a
+// call: inlined, the compiler computes its FP64 operations for every value and
+// selects, 345 -> 544 us for the links of 12^3 x 16); marks *bad if a left the range
+static __device__ __noinline__ float scaled_below(float hi, float lo, int e)
+{
+    return (float)(((double)hi + (double)lo) * (double)pow2f(-e));
+}
+__device__ __forceinline__ float scaled_out(dfl a, int e, int* bad)
+{
+    if (!in_range(a.hi)) *bad = 1;
+    const float r = a.hi * pow2f(-e);
+    return fabsf(r) < 1.17549435e-38f && a.hi != 0.f ? scaled_below(a.hi, a.lo, e) : r;
+}
 template <typename A, typename B> __device__ __forceinline__ void cmacc(cx<A> x, cx<B> y, cx<A>& acc)
 {
     macc(x.re, y.re, acc.re);
@@ -181,10 +209,10 @@ template <typename A> __device__ __forceinline__ void mm_acc(const cx<A>* X, con
 #endif   // __CUDACC__
 
 // the 40 transporters from V64 ([4][9][site], FP64) into W [40][9][site]: FP64,
-// or double-float when df
+// or double-float when df (W of k hops times 2^(k DF_V))
 cudaError_t launch_build_W(const Geom& g, const void* V64, void* W, bool df, cudaStream_t st);
-// nmat matrices per site from a double-float field [m][9][site] into storage
-// precision (blocked layout)
-cudaError_t launch_convert_links_df(int prec, const Geom& g, int nmat, const void* src, void* dst, cudaStream_t st);
+// the 40 double-float transporters into storage precision (blocked layout); *bad
+// is set where one is not finite
+cudaError_t launch_convert_W_df(int prec, const Geom& g, const void* W, void* dst, int* bad, cudaStream_t st);
 
 }  // namespace dirac
