@@ -184,7 +184,8 @@ DIRAC_API dirac_status dirac_apply_dagger(dirac_handle* h, void* out, const void
  *   G_dir(y) = sum_v,s g_v(y)_s (M_dir psi_v(y+dir))_s^+ is passed down the
  *   recursion W_dir(x) = (1/k) sum_a H_a(x) W_{dir-a}(x+a) to the links.
  *   Takes scratch of 121 * 9 complex doubles per site (17.4 KB per site) during
- *   the call; up to 1 GiB of it stays with the handle for the next call.
+ *   the call; up to 1 GiB of it stays with the handle for the next one, until another
+ *   allocation of the handle finds no memory.
  *   F        device, canonical link layout [s][mu][a][b], complex double for
  *            F64 handles and complex float otherwise; written once per link
  *   psi, g   device spinor fields in `layout`

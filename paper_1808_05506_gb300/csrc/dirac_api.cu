@@ -58,6 +58,12 @@ dirac_status dirac_handle::alloc(void** p, size_t bytes, const char* what)
     *p = nullptr;
     if (bytes == 0) return DIRAC_OK;
     cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && scr && !scr_busy) {   // give the kept scratch back
+        cudaGetLastError();
+        release(scr);
+        scr_bytes = 0;
+        e = cudaMalloc(p, bytes);
+    }
     if (e != cudaSuccess) {
         *p = nullptr;
         cudaGetLastError();
@@ -361,7 +367,7 @@ dirac_status dirac_set_links(dirac_handle* h, const void* V, dirac_prec V_prec, 
             // W rounded to FP32 or less: built in double-float (the solver builds FP64 W on demand),
             // again in FP64 if an entry left the range
             void* W = nullptr;
-            if ((st = h->scratch((size_t)h->g.vol * 40 * 9 * 16, &W))) return st;
+            if ((st = h->scratch((size_t)h->g.vol * 40 * 9 * 16, false, &W))) return st;
             // the FP32 copy of the split inner solve is refreshed in place (a
             // captured solver graph holds its address)
             void* L32 = h->links32 != h->links ? h->links32 : nullptr;
@@ -524,12 +530,13 @@ dirac_status dirac_handle::build_W64()
     return st;
 }
 
-// scratch of the W build and of the Brillouin link gradient (17 KB per site).
-// Up to SCRATCH_KEEP bytes stay with the handle for the next call: allocating
-// and freeing 0.5 GB took 1.4 ms of a 2.6 ms gradient (12^3 x 16).  A larger one is
-// given back after the call.  scratch_done waits for the stream, so a later
-// call may use the memory on another one.
-dirac_status dirac_handle::scratch(size_t bytes, void** out)
+// scratch of the W build (5.8 KB per site) and of the Brillouin link gradient (17.4 KB).
+// What a gradient took stays with the handle for the next one, up to SCRATCH_KEEP bytes (61 600
+// sites): allocating and freeing 0.5 GB took 1.4 ms of a 2.6 ms gradient (12^3 x 16).  A larger
+// one, and that of a handle that has taken no gradient, is given back after the call, and
+// a kept one when another allocation of the handle finds no memory.
+// scratch_done waits for the stream, so a later call may use the memory on another one.
+dirac_status dirac_handle::scratch(size_t bytes, bool keep, void** out)
 {
     if (bytes > scr_bytes) {
         release(scr);
@@ -538,6 +545,8 @@ dirac_status dirac_handle::scratch(size_t bytes, void** out)
         if (st) return st;
         scr_bytes = bytes;
     }
+    scr_keep = scr_keep || keep;
+    scr_busy = true;
     *out = scr;
     return DIRAC_OK;
 }
@@ -545,7 +554,8 @@ dirac_status dirac_handle::scratch(size_t bytes, void** out)
 void dirac_handle::scratch_done()
 {
     cudaStreamSynchronize(stream);
-    if (scr_bytes > SCRATCH_KEEP) {
+    scr_busy = false;
+    if (!scr_keep || scr_bytes > SCRATCH_KEEP) {
         release(scr);
         scr_bytes = 0;
     }

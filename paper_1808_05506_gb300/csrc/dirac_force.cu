@@ -255,7 +255,7 @@ static dirac_status force_internal(dirac_handle* h, void* F, const void* pi, con
     const size_t plane = (size_t)h->g.vol * 9 * 16;
     void* scr = nullptr;
     dirac_status st;
-    if ((st = h->scratch(121 * plane, &scr))) return st;
+    if ((st = h->scratch(121 * plane, true, &scr))) return st;
     auto run = [&](bool f64) {
         return h->cuda(launch_force_brillouin(h->prec, f64, h->g, h->Nv, pi, gi, h->links64, scr,
                                               static_cast<char*>(scr) + 40 * plane, F, h->range_flag, h->stream),

@@ -47,6 +47,8 @@ struct dirac_handle {
     static constexpr size_t SCRATCH_KEEP = (size_t)1 << 30;
     void* scr = nullptr;      // scratch of the W build and the Brillouin link gradient
     size_t scr_bytes = 0;
+    bool scr_keep = false;    // a gradient was taken: its scratch stays
+    bool scr_busy = false;    // between scratch and scratch_done
     int* range_flag = nullptr;   // device word: a double-float chain left FP32's range (dirac_transport.cuh)
 
     // solver workspace (dirac_solve.cu)
@@ -71,7 +73,7 @@ struct dirac_handle {
     double diag_of(double mass) const;
     dirac_status ensure_workspace();
     dirac_status build_W64();
-    dirac_status scratch(size_t bytes, void** out);
+    dirac_status scratch(size_t bytes, bool keep, void** out);
     void scratch_done();
     dirac_status clear_range_flag();
     dirac_status read_range_flag(bool* left);   // waits for the stream
