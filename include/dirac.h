@@ -413,8 +413,11 @@ DIRAC_API dirac_status dirac_get_kernel_config(const dirac_handle* h, int* R, in
  *                 the t-neighbours of a site are swept a few planes after it
  *                 and are still in L2 (with 12 FP32 right-hand sides a 32^3
  *                 t-slice and its output are larger than half the L2).
- * Results do not depend on it.  Kept across dirac_set_kernel_config; chosen
- * by dirac_autotune.  INVALID_ARG outside 0..Nt. */
+ * Results do not depend on it.  Chosen by dirac_autotune; a handle that was not
+ * tuned starts with tchunk = min(8, Nt) where a t-slice of one field takes more than
+ * 25 MB (Wilson and staggered, FP32 and 16-bit), else with 0.  Kept across
+ * dirac_set_kernel_config once it was set or tuned; until then a shape set by hand is
+ * lexicographic.  INVALID_ARG outside 0..Nt. */
 DIRAC_API dirac_status dirac_set_site_order(dirac_handle* h, int tchunk);
 DIRAC_API dirac_status dirac_get_site_order(const dirac_handle* h, int* tchunk);
 

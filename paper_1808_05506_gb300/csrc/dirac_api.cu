@@ -664,7 +664,8 @@ dirac_status dirac_set_kernel_config(dirac_handle* h, int R, int block, int vari
         const dirac_status st = dirac_set_link_format(h, 1);
         if (st) return st;
     }
-    h->cfg = LaunchCfg{R, block, variant, h->cfg.order};
+    // a site order that was set or tuned is kept, the default shape's is not
+    h->cfg = LaunchCfg{R, block, variant, h->order_set ? h->cfg.order : 0};
     return DIRAC_OK;
 }
 
@@ -707,6 +708,7 @@ dirac_status dirac_set_site_order(dirac_handle* h, int tchunk)
         return h->fail(DIRAC_ERR_INVALID_ARG, "dirac_set_site_order: tchunk = %d not in 0..Nt = %d", tchunk,
                        h->g.L[3]);
     h->cfg.order = tchunk;
+    h->order_set = true;
     return DIRAC_OK;
 }
 

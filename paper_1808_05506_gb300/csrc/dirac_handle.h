@@ -18,6 +18,7 @@ struct dirac_handle {
     cudaStream_t stream = nullptr;
     int device = 0;
     dirac::LaunchCfg cfg{1, 128, dirac::V_DIRECT};
+    bool order_set = false;   // cfg.order was set by hand or by the tuner (not the default's)
     int precond = 1;          // inner solves: 1 even-odd where it applies, 0 whole lattice
     int outer_df = 1;         // outer residual: 1 double-float sweep (non-FP64 handles), 0 FP64
     int inner_fields = 1;     // 16-bit Wilson even-odd inner solves: 1 split fields, 0 all 16-bit

@@ -172,6 +172,7 @@ extern "C" DIRAC_API dirac_status dirac_autotune(dirac_handle* h, int force, int
     if (!force && cache_lookup(key, &R, &B, &Pp, &Tc, &best, &Fm) &&
         apply_config_supported(h->op, h->prec, R, B, Pp, h->g) && Tc >= 0 && Tc <= h->g.L[3]) {
         h->cfg = LaunchCfg{R, B, Pp, Tc};
+        h->order_set = true;
         // the cached link format, if these links allow it
         if (dirac_set_link_format(h, Fm) != DIRAC_OK) dirac_set_link_format(h, 0);
     } else {
@@ -266,6 +267,7 @@ extern "C" DIRAC_API dirac_status dirac_autotune(dirac_handle* h, int force, int
             return st;
         }
         h->cfg = LaunchCfg{win.R, win.block, win.variant, win.order};
+        h->order_set = true;
         h->link_fmt = win.fmt == 1 ? 1 : 0;
         if (h->link_fmt == 0) h->release_link_alt();
         cache_store(key, win.R, win.block, win.variant, win.order, best, h->link_fmt);

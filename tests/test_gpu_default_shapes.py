@@ -36,3 +36,14 @@ def test_default_site_order(dg, L, Nv):
     for a, b in zip(order[8], order[0]):
         assert torch.equal(torch.view_as_real(a), torch.view_as_real(b))
     D.close()
+
+
+def test_shape_set_by_hand_starts_lexicographic(dg):
+    D = dg.Dirac("wilson", (16, 16, 16, 10), 64, 0.12, "f32")
+    assert D.site_order() == 8
+    D.set_kernel_config(2, 64, 1)
+    assert D.site_order() == 0
+    D.set_site_order(3)
+    D.set_kernel_config(1, 128, 0)
+    assert D.site_order() == 3
+    D.close()
