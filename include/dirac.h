@@ -189,14 +189,16 @@ DIRAC_API dirac_status dirac_apply_dagger(dirac_handle* h, void* out, const void
  *   F        device, canonical link layout [s][mu][a][b], complex double for
  *            F64 handles and complex float otherwise; written once per link
  *   psi, g   device spinor fields in `layout`
- * Asynchronous. */
+ * Brillouin requires dirac_set_links first (else INVALID_ARG) and waits for the
+ * stream; Wilson and staggered are asynchronous and do not read the links. */
 DIRAC_API dirac_status dirac_force(dirac_handle* h, void* F, const void* psi, const void* g,
                                    dirac_layout layout);
 
 /* The whole backward pass of out = D psi for the cotangent g: gpsi = D^+ g
  * (dirac_apply_dagger) and F (dirac_force), with g converted to the internal
- * layout once.  All fields canonical, device; no two may be the same.
- * Asynchronous. */
+ * layout once.  All fields canonical, device; gpsi and F may be neither input nor
+ * each other.  Requires dirac_set_links first.  Asynchronous, except for Brillouin,
+ * which waits for the stream. */
 DIRAC_API dirac_status dirac_backward(dirac_handle* h, void* gpsi, void* F, const void* psi, const void* g);
 
 /* Statistics of one dirac_solve call. */

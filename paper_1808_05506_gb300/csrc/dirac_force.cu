@@ -250,6 +250,8 @@ static dirac_status force_internal(dirac_handle* h, void* F, const void* pi, con
 {
     if (h->op != OP_BRILLOUIN)
         return h->cuda(launch_force(h->op, h->prec, h->g, h->Nv, pi, gi, F, h->stream), "force kernel launch");
+    if (!h->have_links)   // Wilson and staggered forces need none
+        return h->fail(DIRAC_ERR_INVALID_ARG, "dirac_force: the Brillouin gradient needs links: call dirac_set_links first");
     // the transporters are rebuilt from V (not kept from the forward pass): 40
     // planes of W and 81 of G
     const size_t plane = (size_t)h->g.vol * 9 * 16;

@@ -73,3 +73,18 @@ def test_force_links_per_thread(dg, op, prec, L, Nv):
     err = ((got - want).abs().square().sum((0, 1, 2, 3, 5, 6)) / want.abs().square().sum((0, 1, 2, 3, 5, 6))).sqrt()
     assert err.max().item() <= TOL[prec], err
     D.close()
+
+
+def test_force_without_links(dg):
+    """Wilson and staggered forces do not read the links; the Brillouin gradient
+    refuses a handle that has none."""
+    L, Nv = (4, 2, 3, 2), 2
+    for op in ("wilson", "staggered", "brillouin"):
+        D = dg.Dirac(op, L, Nv, 0.12, "f32")
+        psi = torch.ones(D.canonical_shape, dtype=torch.complex64, device="cuda")
+        if op == "brillouin":
+            with pytest.raises(dg.DiracError, match="dirac_set_links"):
+                D.force(psi, psi)
+        else:
+            assert torch.isfinite(torch.view_as_real(D.force(psi, psi))).all()
+        D.close()
