@@ -453,9 +453,6 @@ class Dirac:
 
     def backward(self, psi, g):
         """(D^+ g, link gradient of Re <g, D psi>), as apply_dagger(g) and force(psi, g) give them."""
-        cls = type(self)
-        if cls.apply_dagger is not Dirac.apply_dagger or cls.force is not Dirac.force or cls.apply is not Dirac.apply:
-            return self.apply_dagger(g), self.force(psi, g)   # a subclass's own
         psi = self._canon_in(psi, "psi")
         g = self._canon_in(g, "g")
         gpsi, F = self.new_canonical(), self._links_out()

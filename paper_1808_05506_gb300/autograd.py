@@ -9,7 +9,7 @@ backward: dL/dpsi = D^+ g (dirac_apply_dagger) and dL/dV = the link force
           gradients are exactly D^+ g and F.
 
 Loading the links into the handle (dirac_set_links: a conversion and, for
-Brillouin, the FP64 build of W) is skipped where it would load what is
+Brillouin, the build of W) is skipped where it would load what is
 already there:
   - backward reloads V only if the handle was given other links after this
     node's forward pass (autograd itself rejects a V changed in place since);
@@ -47,14 +47,21 @@ class DiracApply(torch.autograd.Function):
         if D.links_generation != ctx.links_generation:
             D.set_links(V)   # the handle was given other links since the forward pass
         gpsi = gV = None
-        if ctx.needs_input_grad[0] and ctx.needs_input_grad[1]:
+        if ctx.needs_input_grad[0] and ctx.needs_input_grad[1] and _own_calls(D):
             gpsi, gV = D.backward(psi.detach(), g)
-            gpsi, gV = gpsi.to(psi.dtype), gV.to(V.dtype)
-        elif ctx.needs_input_grad[0]:
+            return gpsi.to(psi.dtype), gV.to(V.dtype), None, None
+        if ctx.needs_input_grad[0]:
             gpsi = D.apply_dagger(g).to(psi.dtype)
-        elif ctx.needs_input_grad[1]:
+        if ctx.needs_input_grad[1]:
             gV = D.force(psi.detach().to(D.canon_dtype).contiguous(), g).to(V.dtype)
         return gpsi, gV, None, None
+
+
+def _own_calls(D) -> bool:
+    """Whether D is a Dirac with the class's own calls, so that its fused backward gives what
+    they give: not a subclass's or one handle's replacements, nor another object that has the
+    calls."""
+    return type(D) is Dirac and not {"apply", "apply_dagger", "force", "backward"} & D.__dict__.keys()
 
 
 def dirac_apply(D: Dirac, psi: torch.Tensor, V: torch.Tensor, reuse_links: bool = True) -> torch.Tensor:
