@@ -196,6 +196,7 @@ class Dirac:
         if getattr(self, "h", None):
             lib().dirac_destroy(self.h)
             self.h = None
+            self.__dict__.pop("_nbytes", None)   # a closed handle has no field size
 
     def __del__(self):
         try:
