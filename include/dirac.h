@@ -69,7 +69,7 @@ typedef enum {
     DIRAC_ERR_CUDA = 4,          /* a CUDA runtime call failed */
     DIRAC_NOT_CONVERGED = 5,     /* solver hit its iteration limit */
     DIRAC_BREAKDOWN = 6,         /* solver met a zero/NaN/Inf scalar */
-    DIRAC_TIMEOUT = 7            /* a bounded device-side wait ran out */
+    DIRAC_TIMEOUT = 7            /* a bounded device-side wait ran out (no kernel has one at present) */
 } dirac_status;
 
 typedef enum { DIRAC_STAGGERED = 0, DIRAC_WILSON = 1, DIRAC_BRILLOUIN = 2 } dirac_op;
@@ -468,10 +468,7 @@ DIRAC_API dirac_status dirac_get_link_format(const dirac_handle* h, int* fmt);
  * and its median time per sweep in milliseconds (from the cache when reused). */
 DIRAC_API dirac_status dirac_autotune(dirac_handle* h, int force, int* R, int* block, int* variant, double* ms);
 
-/* Wait for the handle's stream and report kernel-side failures: returns
- * DIRAC_TIMEOUT (and clears the record) if a kernel recorded that a bounded
- * device-side wait ran out since the last call (no kernel built at present
- * has one), else DIRAC_OK or the CUDA error of the stream. */
+/* Wait for the handle's stream: DIRAC_OK or the CUDA error of the stream. */
 DIRAC_API dirac_status dirac_sync(dirac_handle* h);
 
 /* One-line description of the last error on h (or of the last failed

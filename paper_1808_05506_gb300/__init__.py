@@ -526,8 +526,7 @@ class Dirac:
         return R.value, B.value, Pp.value, ms.value
 
     def sync(self):
-        """Wait for the handle's stream; raises DiracError(TIMEOUT) if a kernel's
-        bounded wait ran out."""
+        """Wait for the handle's stream."""
         check(lib().dirac_sync(self.h), self.h, "dirac_sync")
 
     def kernel_config(self):

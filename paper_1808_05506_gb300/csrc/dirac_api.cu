@@ -123,7 +123,6 @@ ApplyArgs dirac_handle::args(void* out, const void* in, int nv, double diag_valu
     a.diag_v = nullptr;
     a.diagf = (float)diag_value;
     a.diag_vf = nullptr;
-    a.err = dev_err;
     a.tc = 0;
     a.t0 = 0;
     a.nt = g.L[3];
@@ -152,7 +151,6 @@ dirac_status dirac_handle::run_apply(bool dagger, void* out, const void* in, int
     a.diag_v = diag_v;
     a.diag_vf = diag_vf;
     a.canon = canon;
-    a.err = dev_err;
     if (nt > 0) {   // the slab of nt t-slices from t0 (variants 0, 1, 2 and 5)
         a.t0 = t0;
         a.nt = nt;
@@ -247,12 +245,6 @@ dirac_status dirac_create(dirac_handle** h, dirac_op op, int Nc, int Nx, int Ny,
         return DIRAC_ERR_CUDA;
     }
     H->cfg = default_config(H->op, H->prec, Nv, &H->g);
-    if (cudaMalloc((void**)&H->dev_err, sizeof(int)) != cudaSuccess || cudaMemset(H->dev_err, 0, sizeof(int)) != cudaSuccess) {
-        cudaGetLastError();
-        g_create_error = "dirac_create: cannot allocate the device error word";
-        delete H;
-        return DIRAC_ERR_OOM;
-    }
     if (H->op == OP_BRILLOUIN) {
         cudaError_t e = upload_brillouin_table(H->stream);
         if (e == cudaSuccess && (prec == DIRAC_BF16 || prec == DIRAC_F16)) e = brillouin_tc_prepare(H->stream);
@@ -269,9 +261,7 @@ dirac_status dirac_create(dirac_handle** h, dirac_op op, int Nc, int Nx, int Ny,
 
 dirac_handle::~dirac_handle()
 {
-    void* e = dev_err;
-    release(e);
-    e = range_flag;
+    void* e = range_flag;
     release(e);
     release(links);
     release(links64);
@@ -779,15 +769,7 @@ dirac_status dirac_get_kernel_config(const dirac_handle* h, int* R, int* block, 
 dirac_status dirac_sync(dirac_handle* h)
 {
     if (!h) return DIRAC_ERR_INVALID_ARG;
-    dirac_status st = h->cuda(cudaStreamSynchronize(h->stream), "dirac_sync");
-    if (st) return st;
-    int e = 0;
-    if ((st = h->cuda(cudaMemcpy(&e, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost), "dirac_sync"))) return st;
-    if (e) {
-        cudaMemset(h->dev_err, 0, sizeof(int));
-        return h->fail(DIRAC_TIMEOUT, "dirac_sync: a kernel's bounded wait ran out (status %d)", e);
-    }
-    return DIRAC_OK;
+    return h->cuda(cudaStreamSynchronize(h->stream), "dirac_sync");
 }
 
 const char* dirac_last_error(const dirac_handle* h)

@@ -39,7 +39,6 @@ struct dirac_handle {
                                 // tensor-core sweep (which reads this copy)
     int link_fmt = 0;           // the format the apply sweeps read where their variant supports it
     bool have_links = false;
-    int* dev_err = nullptr;   // device error word written by kernels whose bounded waits run out
 
     void* ws_in = nullptr;    // internal-layout workspaces of the canonical apply
     void* ws_out = nullptr;

@@ -40,7 +40,6 @@ struct ApplyArgs {
     const double* diag_v; // per-right-hand-side diagonal (device, Nv entries) or null: diag for all
     float diagf;          // the same in FP32, for the FP32-arithmetic sweeps (no FP64
     const float* diag_vf; // conversion inside them)
-    int* err;             // device error word (kernels with bounded waits record DIRAC_TIMEOUT) or null
     int tc;               // site order of the grid (site_of): 0 lexicographic, else t-chunk
     // the sweep covers the slab of nt t-slices starting at slice t0 (sites
     // t0 Lx Ly Lz .. + nsites); the whole lattice: t0 = 0, nt = Nt

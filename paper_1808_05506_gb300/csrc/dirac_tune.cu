@@ -189,10 +189,9 @@ extern "C" DIRAC_API dirac_status dirac_autotune(dirac_handle* h, int force, int
             return st;
         }
         // median of 5 timed calls after 2 warm-up calls; false if the shape
-        // cannot run here or a kernel recorded a failure (never picked)
+        // cannot run here (never picked)
         auto time_cfg = [&](const LaunchCfg& c, double* med) -> bool {
             std::vector<float> t;
-            cudaMemsetAsync(h->dev_err, 0, sizeof(int), h->stream);
             for (int rep = 0; rep < 7 && st == DIRAC_OK; ++rep) {
                 cudaEventRecord(e0, h->stream);
                 const dirac_status ls = h->run_apply(false, h->ws_out, h->ws_in, h->Nv, h->diag, h->links, h->prec, c);
@@ -207,12 +206,6 @@ extern "C" DIRAC_API dirac_status dirac_autotune(dirac_handle* h, int force, int
                 if (rep >= 2) t.push_back(ms);   // two warm-up calls
             }
             if (st) return false;
-            int kerr = 0;
-            cudaMemcpy(&kerr, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost);
-            if (kerr) {
-                cudaMemset(h->dev_err, 0, sizeof(int));
-                return false;
-            }
             std::sort(t.begin(), t.end());
             *med = t[t.size() / 2];
             const char* tr = getenv("DIRAC_TRACE");
