@@ -400,7 +400,9 @@ DIRAC_API dirac_status dirac_get_residual_arithmetic(const dirac_handle* h, int*
  *               afterwards; one CTA per SM works on tiles of up to 16 sites of an
  *               (x, y) plane (up to 227 KB of shared memory).  The C_j are
  *               powers of two up to a factor per class, so the C_j W are exact
- *               in 16 bits.  Selecting it selects link format 1.
+ *               in BF16; in FP16 those below 2^-14 (|W| < 2^-8 at four hops) are
+ *               rounded to 2^-25, at most 2^-19 of W.  Selecting it selects link
+ *               format 1.
  * UNSUPPORTED for other values. */
 DIRAC_API dirac_status dirac_set_kernel_config(dirac_handle* h, int R, int block, int variant);
 

@@ -8,8 +8,10 @@
 //   D_B psi_v(x)[s] = (m0 + 15/8) psi_v(x)[s] + T_0[s] + sum_mu (gamma_mu T_{1+mu})[s].
 // The coefficients are powers of two up to one factor per class kind,
 //   C_0 = -(1/16) 2^(1-k),   C_{1+mu} = (4/27) d_mu 4^(1-k),
-// so the products C W are formed exactly in 16 bits (the factors go into the
-// epilogue) and the only rounding before the FP32 sums is that of the stored W.
+// so the products C W are formed in 16 bits (the factors go into the epilogue),
+// exactly in BF16, so that the only rounding before the FP32 sums is that of the stored
+// W.  In FP16 products below 2^-14 (|W| < 2^-8 at four hops, 2^-11 in C_0) are rounded to
+// 2^-25, which is at most 2^-19 of W, next to 2^-12 for an entry near 1.
 //
 // One warp owns a site and up to 16 right-hand sides: a real matrix product
 //   T[(j, c, re/im)][(s, v)] = A[(j, c, re/im)][(d, c', re/im)] B[(d, c', re/im)][(s, v)]
@@ -37,7 +39,7 @@
 // building those in 4- and 8-byte stores (6900 instructions and 1600 wavefronts per
 // site) bounded that kernel.  16^3 x 32, BF16, one GB300: Nv = 16: 1.85 ms
 // with tcgen05 and on CUDA cores, 1.17 ms here; Nv = 12: 1.45 ms on CUDA
-// cores, 1.00 ms; Nv = 4: 0.54 and 0.51 ms.
+// cores, 0.95 ms; Nv = 4: 0.54 and 0.51 ms.
 #include <algorithm>
 #include <mutex>
 
